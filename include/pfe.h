@@ -55,7 +55,8 @@ typedef enum {
 #define PFE_SKIP_SYM_CHECK 0x2u /* do not verify the symmetry of Delta */
 
 /* element types of pfe_filter_apply's X and Y */
-#define PFE_F64 0 /* float64 vectors, float64 arithmetic */
+#define PFE_F64 0 /* float64 vectors, at least float64 accuracy (64-bit fixed point with a scale per column and
+                     step where the operator fits, else float64 arithmetic) */
 #define PFE_F32 1 /* float32 vectors, float32 arithmetic (mixed-precision filter) */
 
 /* parameter keys for pfe_set_param / pfe_get_param (values are doubles) */
@@ -84,7 +85,8 @@ enum {
   PFE_P_COUNT_DAMPING = 16, /* damping of the estimator series (default 0: plain truncation) */
   PFE_P_MIN_WIDTH = 17,     /* lower bound on the automatic width (default 16) */
   PFE_P_REFINE_TOL = 18,    /* mixed mode: residual below which a pair's filter runs in FP64 (default 1e-4) */
-  PFE_P_STEP_SHAPE_F64 = 19, /* PROCESS-WIDE: kernel shape of the FP64 filter step, -1 = autotuned (default),
+  PFE_P_STEP_SHAPE_F64 = 19, /* PROCESS-WIDE: kernel shape of the FP64 filter step, -1 = automatic (default: the
+                               fixed-point step, reported as 12, where the operator fits, else autotuned),
                                0 warp per (atom, column chunk), 1 CTA per 8 atoms x chunk, 2 and 3: the
                                same with two 3x3 blocks in flight per iteration, 4: neighbour rows staged
                                in shared memory by cp.async four blocks ahead (16-byte lanes), 5 and 6:
@@ -251,7 +253,7 @@ typedef struct {
   int32_t restarts;            /* METHOD 1: thick restarts */
   int32_t basis;               /* METHOD 1: maximal basis size */
   int32_t filter_shape_f64;    /* kernel shape of the last FP64 filter step (PFE_P_STEP_SHAPE_F64 numbering;
-                                  7-9: the rank-1 form), -1 if none ran */
+                                  7-9: the rank-1 form; 12: fixed point), -1 if none ran */
   int32_t filter_shape_f32;    /* the same for the FP32 filter step */
   int32_t slices;              /* pfe_solve_sliced: number of slices (0 for the other solves) */
   int32_t active;              /* stepwise solve in progress: columns still iterating (0 otherwise) */
@@ -315,8 +317,9 @@ pfe_status pfe_chain_springs(pfe_ctx *ctx, int64_t nbonds, const int32_t *bi, co
  * coeffs: host array of m + 1 coefficients (required); X, Y: device pointers, column-major n x k,
  * ld >= n, float64; stream as in pfe_filter_apply.  Given a stream other than the context's, the
  * call first waits on the host for the context's stream, where the filter operator was built.
- * It runs the kernel shape that pfe_filter_apply tuned for this column count (shape 0 before any
- * tuning), and does not time shapes itself. */
+ * It runs the kernel that pfe_filter_apply runs, with the fixed-point operator if an earlier FP64 filter call built
+ * it, else the FP64 shape tuned for this column count (0, or 7 on the rank-1 form, before any tuning), and does not
+ * time shapes itself. */
 pfe_status pfe_filter_apply_noalloc(pfe_ctx *ctx, int32_t m, const double *coeffs, int32_t k, const double *X,
                                     int64_t ldx, double *Y, int64_t ldy, void *stream);
 

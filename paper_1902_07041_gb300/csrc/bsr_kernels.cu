@@ -313,7 +313,9 @@ bool aligned(const void *p, size_t a) { return p == nullptr || (reinterpret_cast
 // run on the rank-1 form of the operator when it has one (r1_kernels.cu: warp per (atom, chunk);
 // five resident CTAs; two blocks in flight); without it they fall back to shape 0.
 // A forced shape (set_step_variant) wins; otherwise the autotuner's choice for (type, columns per
-// lane, column chunks, rank-1 form present) is used, and the default 0 before any tuning.
+// lane, column chunks, rank-1 form present) is used, and before any tuning 7 on the rank-1 form, else 0.
+// The FP64 filter itself runs in fixed point (fixed_step.cu) unless a shape is forced; these FP64 shapes serve the
+// adjoint, products with H and operators that do not fit.
 namespace {
 // The tuner times the full-block shapes 0-6, or the rank-1 shapes 7-9 when the operator has that form.
 // Shape 10 (FP32, rows staged in shared memory) runs only when forced: it measured 3.6x slower than
@@ -329,7 +331,7 @@ int pick_variant(int is_float, int cpl, int32_t nchunk, bool r1) {
   if (g_forced[is_float] >= 0) return g_forced[is_float];
   std::lock_guard<std::mutex> lk(g_tune_mu);
   auto it = g_tuned.find(std::make_tuple(is_float, cpl, std::min(nchunk, 16), r1 ? 1 : 0));
-  return it == g_tuned.end() ? 0 : it->second;
+  return it == g_tuned.end() ? (r1 ? kVariants : 0) : it->second;
 }
 }  // namespace
 

@@ -1,0 +1,757 @@
+// The FP64 filter (Alg. 2) in 64-bit fixed point.
+//
+// Why: GB300 issues 2 FP64 FMAs a clock and SM, but about 30 32 x 32 + 64-bit multiply-adds (IMAD.WIDE, measured)
+// and 64 to 128 of the simpler integer operations.  A multiply-add of two 60-bit numbers is three IMAD.WIDE, a
+// fifth of the time of one FP64 FMA, and the step leaves the FP64 pipe, where it ran at 0.9 of its rate.
+//
+// Numbers.  A Chebyshev vector is stored as (h, l) pairs of int32: value (h 2^30 + l) 2^-sh with l in
+// [-2^29, 2^29) and one exponent sh per column and vector; |h| <= 2^30.  The operator A = (2/d)(H - cI) is stored
+// in the same split, U = u 2^60 = uh 2^30 + ul (full blocks: a 2^59).  A product keeps
+//   uh xh 2^60 + (uh xl + ul xh) 2^30     (two 64-bit sums, accH and accM; ul xl 2^-60 <= 2^-2 of a unit is dropped)
+// and a sum over a row is rounded once, (accH + (accM + 2^29) >> 30), in units of the input vector.  A column's
+// largest entry times ||A||_inf + 1 fills 60 bits, so for ||A||_inf near 6 a typical entry has 55 bits, and a step
+// adds about half a unit of rounding to it, 2^-56: the FMA chain of a row takes 13 to 40 roundings of 2^-53.
+// Measured against 128-bit arithmetic with the same operator (relative 2-norm of a column): 0.9e-15 (FP64 kernels
+// 1.6e-15) at degree 40, 1.9e-15 (2.6e-15) at 301, 0.3e-15 (1.4e-15) with full blocks.  Errors are relative to a
+// column's largest entry, as the recurrence mixes the entries of a column.
+//
+// Scaling.  Each step knows, per column, bounds M on the |h| of t_j and t_{j-1} and the exponents, so every CTA
+// derives the same shift o of the new vector from
+//   |t_{j+1}| <= ||A||_inf |t_j| + |t_{j-1}|  <  2^60:
+// right when that could overflow, left when two or more bits would lie idle.  In a filter whose spectrum lies
+// in [-1, 1] the shift is almost always 0; vectors that grow (a bound below the spectrum) or spread (a start
+// concentrated on few atoms) move their exponent.  M of the new vector is an atomic maximum that starts at 1/16
+// of a recent one, so that few lanes write.  State: 4 rotating slots of sh and M per column.
+//
+// Columns with an Inf, a NaN or entries beyond 2^+-900 keep doubles in the same buffers and take the FP64 FMAs
+// inside the same kernel (kRaw), so every input gives what it gave before.
+#include <cmath>
+
+#include "pfe_internal.h"
+
+namespace pfe {
+namespace {
+
+constexpr int kLimb = 30;                    // bits of the low limb
+constexpr int32_t kMask = (1 << kLimb) - 1;  // low limb of a non-negative remainder
+constexpr int32_t kHalf = 1 << (kLimb - 1);
+constexpr int32_t kRaw = INT32_MIN;          // exponent of a column kept in FP64
+
+// The full product.  As assembly with the addition outside it becomes one multiply-add; the C product of two
+// loaded words becomes three multiplies, and mad.wide a multiply and a separate addition (2.8 x, 1.5 x the
+// instructions of a block).
+__device__ __forceinline__ int64_t mul(int32_t a, int32_t b) {
+  int64_t d;
+  asm("mul.wide.s32 %0, %1, %2;" : "=l"(d) : "r"(a), "r"(b));
+  return d;
+}
+__device__ __forceinline__ int64_t mad(int32_t a, int32_t b, int64_t c) { return mul(a, b) + c; }
+
+// (h, l) of a 64-bit value: h rounded to nearest, l the signed rest
+__device__ __forceinline__ int2 split(int64_t v) {
+  const int64_t t = v + kHalf;
+  return make_int2((int32_t)((uint32_t)t & kMask) - kHalf, (int32_t)(t >> kLimb));
+}
+__device__ __forceinline__ int64_t join(int2 p) { return mad(p.y, 1 << kLimb, (int64_t)p.x); }
+// v 2^o, rounded to nearest for o < 0
+__device__ __forceinline__ int64_t shifted(int64_t v, int o) {
+  if (o >= 0) return o > 62 ? 0 : (int64_t)((uint64_t)v << o);
+  return o < -62 ? 0 : (v + ((int64_t)1 << (-o - 1))) >> -o;
+}
+// exact up to one rounding to double; two FP64 additions (the conversion instruction runs at 2 a clock as well)
+__device__ __forceinline__ double to_double(int64_t v) {
+  const uint32_t lo = (uint32_t)v, hi = (uint32_t)((uint64_t)v >> 32) ^ 0x80000000u;
+  const double dl = __hiloint2double(0x43300000, (int)lo);  // 2^52 + lo
+  const double dh = __hiloint2double(0x45300000, (int)hi);  // 2^84 + (hi + 2^31) 2^32
+  return (dh - 0x1.00000801p84) + dl;                      // 2^84 + 2^63 + 2^52
+}
+__device__ __forceinline__ double pow2(int e) {
+  return __hiloint2double(e < -1022 ? 0 : (min(e, 1024) + 1023) << 20, 0);  // 0 and Inf outside the range
+}
+
+template <int CPL>
+__device__ __forceinline__ void load_pairs(const int2 *p, int2 (&v)[CPL]) {
+  if constexpr (CPL == 2) {
+    const int4 t = __ldg(reinterpret_cast<const int4 *>(p));
+    v[0] = make_int2(t.x, t.y);
+    v[1] = make_int2(t.z, t.w);
+  } else {
+    v[0] = __ldg(p);
+  }
+}
+template <int CPL>
+__device__ __forceinline__ void load_own(const int2 *p, int2 (&v)[CPL]) {  // the kernel writes this buffer
+  if constexpr (CPL == 2) {
+    const int4 t = *reinterpret_cast<const int4 *>(p);
+    v[0] = make_int2(t.x, t.y);
+    v[1] = make_int2(t.z, t.w);
+  } else {
+    v[0] = *p;
+  }
+}
+template <int CPL>
+__device__ __forceinline__ void store_pairs(int2 *p, const int2 (&v)[CPL]) {
+  if constexpr (CPL == 2)
+    *reinterpret_cast<int4 *>(p) = make_int4(v[0].x, v[0].y, v[1].x, v[1].y);
+  else
+    *p = v[0];
+}
+template <int CPL>
+__device__ __forceinline__ void load_y(const double *p, double (&v)[CPL]) {
+  if constexpr (CPL == 2) {
+    const double2 t = *reinterpret_cast<const double2 *>(p);
+    v[0] = t.x;
+    v[1] = t.y;
+  } else {
+    v[0] = *p;
+  }
+}
+template <int CPL>
+__device__ __forceinline__ void store_y(double *p, const double (&v)[CPL]) {
+  if constexpr (CPL == 2)
+    *reinterpret_cast<double2 *>(p) = make_double2(v[0], v[1]);
+  else
+    *p = v[0];
+}
+template <int CPL>
+__device__ __forceinline__ void load_state(const int32_t *p, int32_t (&v)[CPL]) {
+  if constexpr (CPL == 2) {
+    const int2 t = *reinterpret_cast<const int2 *>(p);
+    v[0] = t.x;
+    v[1] = t.y;
+  } else {
+    v[0] = *p;
+  }
+}
+
+// arguments of one step (j -> j + 1)
+struct StepArgs {
+  int32_t n_atoms;
+  int32_t groups, tile;      // CPL-wide column groups per row; of them per CTA
+  int32_t per_pass, passes;  // atoms of a CTA at a time, and how often
+  uint32_t magic;            // division of a lane's slot by tile: (slot magic) >> 16
+  int64_t ld;
+  const int32_t *rp;     // row starts: off-diagonal blocks (rank-1) or all blocks (full)
+  const int4 *blk;       // rank-1: two int4 per block (u0, u1 | u2, column, 0); full: five (nine pairs, column, 0)
+  const int4 *dg;        // rank-1: six pairs per atom (three int4), negated
+  const double *u64, *d64;  // the same operator in FP64 for the columns kept in FP64
+  const int32_t *ci64;
+  const int32_t *info;   // see note_row
+  const int2 *X, *W;
+  int2 *Z;
+  double *Y;
+  int32_t *sh, *mx;      // [4][kc]
+  int64_t kc;
+  int32_t j;
+  int2 ga, gb;           // g_j, g_{j+1} times 2^(kLimb * 2 - 1 - ge), split
+  int32_t ge;
+  double g0, g1;         // the same coefficients
+};
+
+// The FP64 form of the step for one lane's columns (an input with Inf, NaN or extreme magnitudes).
+template <int CPL, int MODE, bool FULL>
+__device__ __noinline__ void raw_step(const StepArgs &a, int64_t atom, int64_t c0) {
+  const double *X = reinterpret_cast<const double *>(a.X);
+  const double *W = reinterpret_cast<const double *>(a.W);
+  double *Z = reinterpret_cast<double *>(a.Z);
+  for (int c = 0; c < CPL; ++c) {
+    double acc[3] = {0.0, 0.0, 0.0};
+    const double *xo = X + 3 * atom * a.ld + c0 + c;
+    if (!FULL) {
+      const double *d = a.d64 + 6 * atom;
+      const double x0 = xo[0], x1 = xo[a.ld], x2 = xo[2 * a.ld];
+      acc[0] = fma(d[0], x0, fma(d[1], x1, d[2] * x2));
+      acc[1] = fma(d[1], x0, fma(d[3], x1, d[4] * x2));
+      acc[2] = fma(d[2], x0, fma(d[4], x1, d[5] * x2));
+    }
+    for (int p = a.rp[atom]; p < a.rp[atom + 1]; ++p) {
+      const int64_t col = a.ci64[p];
+      const double *x = X + 3 * col * a.ld + c0 + c;
+      const double x0 = x[0], x1 = x[a.ld], x2 = x[2 * a.ld];
+      if (FULL) {
+        const double *v = a.u64 + 9 * (int64_t)p;
+        for (int r = 0; r < 3; ++r) acc[r] = fma(v[3 * r], x0, fma(v[3 * r + 1], x1, fma(v[3 * r + 2], x2, acc[r])));
+      } else {
+        const double *u = a.u64 + 3 * (int64_t)p;
+        const double s = fma(u[0], x0, fma(u[1], x1, u[2] * x2));
+        for (int r = 0; r < 3; ++r) acc[r] = fma(-s, u[r], acc[r]);
+      }
+    }
+    for (int r = 0; r < 3; ++r) {
+      const int64_t off = (3 * atom + r) * a.ld + c0 + c;
+      double z = MODE == MODE_FIRST ? 0.5 * acc[r] : acc[r] - W[off];
+      Z[off] = z;
+      if (MODE == MODE_FIRST) a.Y[off] = fma(a.g1, z, a.g0 * X[off]);
+      else if (MODE == MODE_STEP_ACC) a.Y[off] = fma(a.g0, X[off], fma(a.g1, z, a.Y[off]));
+      else if (a.Y) a.Y[off] = fma(a.g1, z, a.Y[off]);
+    }
+  }
+}
+
+// What the operator allows: the bits of a stored value (64 hold (||A||_inf + 1) of them) and the blocks whose
+// cross terms 64 bits hold.
+__device__ __forceinline__ float norm_of(const int32_t *info) { return fmaxf(__int_as_float(__ldg(info + 1)), 2.f); }
+__device__ __forceinline__ int top_of(float g) { return g < 6.9f ? 60 : g < 14.9f ? 59 : 58; }
+// pairs of rank-1 blocks between two folds
+__device__ __forceinline__ int fold_of(const int32_t *info) {
+  return __int_as_float(__ldg(info + 2)) < 15.5f ? 3 : __int_as_float(__ldg(info + 3)) < 15.5f ? 2 : 1;
+}
+
+template <int CPL>
+__device__ __forceinline__ void load_atom(const char *xl, uint32_t col, uint32_t stride, int64_t ldb, int2 (&x)[3][CPL]) {
+  const char *p = xl + (uint64_t)col * stride;
+  load_pairs<CPL>(reinterpret_cast<const int2 *>(p), x[0]);
+  load_pairs<CPL>(reinterpret_cast<const int2 *>(p + ldb), x[1]);
+  load_pairs<CPL>(reinterpret_cast<const int2 *>(p + 2 * ldb), x[2]);
+}
+
+// accH, accM += (3 x 3 block v) x, v nine pairs
+template <int CPL>
+__device__ __forceinline__ void add_block(const int2 (&v)[9], const int2 (&x)[3][CPL], int64_t (&accH)[3][CPL],
+                                          int64_t (&accM)[3][CPL]) {
+#pragma unroll
+  for (int r = 0; r < 3; ++r)
+#pragma unroll
+    for (int s = 0; s < 3; ++s)
+#pragma unroll
+      for (int c = 0; c < CPL; ++c) {
+        accH[r][c] = mad(v[3 * r + s].y, x[s][c].y, accH[r][c]);
+        accM[r][c] = mad(v[3 * r + s].y, x[s][c].x, accM[r][c]);
+        accM[r][c] = mad(v[3 * r + s].x, x[s][c].y, accM[r][c]);
+      }
+}
+
+// accH, accM += u (u . x)
+template <int CPL>
+__device__ __forceinline__ void add_rank1(const int4 &b0, const int4 &b1, const int2 (&x)[3][CPL],
+                                          int64_t (&accH)[3][CPL], int64_t (&accM)[3][CPL]) {
+  const int2 u[3] = {make_int2(b0.x, b0.y), make_int2(b0.z, b0.w), make_int2(b1.x, b1.y)};
+#pragma unroll
+  for (int c = 0; c < CPL; ++c) {
+    // s = u . x rounded, plus half a limb so that its low limb comes out signed
+    int64_t H = mul(u[0].y, x[0][c].y), M = mad(u[0].y, x[0][c].x, (int64_t)kHalf + ((int64_t)kHalf << kLimb));
+    M = mad(u[0].x, x[0][c].y, M);
+#pragma unroll
+    for (int r = 1; r < 3; ++r) {
+      H = mad(u[r].y, x[r][c].y, H);
+      M = mad(u[r].y, x[r][c].x, M);
+      M = mad(u[r].x, x[r][c].y, M);
+    }
+    const int64_t t = H + (M >> kLimb);
+    const int32_t sl = (int32_t)((uint32_t)t & kMask) - kHalf, s = (int32_t)(t >> kLimb);
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+      accH[r][c] = mad(u[r].y, s, accH[r][c]);
+      accM[r][c] = mad(u[r].y, sl, accM[r][c]);
+      accM[r][c] = mad(u[r].x, s, accM[r][c]);
+    }
+  }
+}
+
+template <int CPL, bool FULL>
+__device__ __forceinline__ void add_neighbour(const int4 *w, const int2 (&x)[3][CPL], int64_t (&accH)[3][CPL],
+                                              int64_t (&accM)[3][CPL]) {
+  if (FULL) {
+    int2 v[9];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      v[2 * t] = make_int2(w[t].x, w[t].y);
+      v[2 * t + 1] = make_int2(w[t].z, w[t].w);
+    }
+    v[8] = make_int2(w[4].x, w[4].y);
+    add_block<CPL>(v, x, accH, accM);
+  } else {
+    add_rank1<CPL>(w[0], w[1], x, accH, accM);
+  }
+}
+
+template <int CPL>
+__device__ __forceinline__ void fold(int64_t (&accH)[3][CPL], int64_t (&accM)[3][CPL]) {
+#pragma unroll
+  for (int r = 0; r < 3; ++r)
+#pragma unroll
+    for (int c = 0; c < CPL; ++c) {
+      accH[r][c] += accM[r][c] >> kLimb;
+      accM[r][c] &= kMask;
+    }
+}
+
+// What a lane needs to know of a column besides its entries
+struct ColumnScale {
+  int32_t o, wsh;  // shift of the new vector; exponent of t_j minus that of t_{j-1}
+  double ysc;      // value of one unit of the filter sum's increment
+};
+
+// One fused step.  A CTA owns `tile` column groups (CPL columns each) and per_pass atoms at a time, a lane one
+// atom and one group; its atoms' blocks (contiguous in the block list) and its columns' scales sit in shared
+// memory, so the neighbour loop's only global loads are the gathers, and passes > 1 spreads the set-up over
+// several atoms.
+// What bounds it: IMAD.WIDE runs at about 30 a clock and SM (measured), 18 a block and column make 165 us of the
+// step at N = 99,900, k = 64, and the moves and additions that share its pipe most of the rest; a step moves 614 MB
+// there, 91 us at 6.76 TB/s.  Measured: 876 -> 303 us a step (k = 64), 13.8 -> 4.75 ms (k = 994), full blocks
+// 250 -> 83 us (N = 20,000, k = 64) against the FP64 kernels.  Three CTAs an SM (80 registers): two hide less of
+// the gathers (321 us), four spill (320 us).  Prefetching the next CTAs' rows into L2 gained nothing (340 us), nor
+// did four lanes an atom where the GPU is not full (N = 1,000, k = 16: 8.9 us either way).
+template <int CPL, int MODE, bool FULL>
+__global__ void __launch_bounds__(256, 3) k_fixed_step(const StepArgs a) {
+  constexpr int kWords = FULL ? 5 : 2;  // int4 per block
+  extern __shared__ int4 smem[];
+  ColumnScale *scale = reinterpret_cast<ColumnScale *>(smem);
+  int4 *sblk = smem + a.tile * CPL;
+  const uint32_t slot = threadIdx.x, mine = (slot * a.magic) >> 16;
+  const int32_t group = blockIdx.y * a.tile + (int32_t)(slot - mine * a.tile);
+  const int32_t c0 = group * CPL;
+  const int32_t first = blockIdx.x * (a.per_pass * a.passes), last = min(first + a.per_pass * a.passes, a.n_atoms);
+  const int sj = a.j & 3, sp = (a.j + 3) & 3, sn = (a.j + 1) & 3, sr = (a.j + 2) & 3;
+  // ---- the blocks of this CTA's atoms, and the scales of its columns
+  const int32_t pbase = __ldg(a.rp + first);
+  {
+    const int32_t words = (__ldg(a.rp + last) - pbase) * kWords;
+    const int4 *src = a.blk + (int64_t)pbase * kWords;
+    for (int32_t t = threadIdx.x; t < words; t += blockDim.x) sblk[t] = __ldg(src + t);
+  }
+  for (int32_t t = threadIdx.x; t < a.tile * CPL; t += blockDim.x) {
+    const int64_t c = (int64_t)blockIdx.y * a.tile * CPL + t;
+    if (c >= a.kc) break;
+    const int32_t mj = a.mx[sj * a.kc + c], shj = a.sh[sj * a.kc + c];
+    const float g = norm_of(a.info);  // >= 2: t_j itself also fits the new scale
+    ColumnScale q{};
+    float bound = g * (float)(mj + 1);
+    bool zero = mj == 0;
+    if (MODE == MODE_FIRST) {
+      bound *= 0.5f;
+    } else {
+      const int32_t mp = a.mx[sp * a.kc + c];
+      q.wsh = shj - a.sh[sp * a.kc + c];
+      bound += (float)(mp + 1) * __int_as_float((min(max(q.wsh, -126), 90) + 127) << 23);
+      zero = zero && mp == 0;
+    }
+    // bound 1.001 < 2^e: room for top - kLimb - e more bits
+    const int e = ((__float_as_int(bound * 1.001f) >> 23) & 255) - 126;
+    const int room = top_of(g) - kLimb - e;
+    q.o = zero ? 0 : room < 0 ? room : room > 1 ? room - 1 : 0;
+    q.ysc = pow2(a.ge + 1 - (shj + q.o));
+    scale[t] = q;
+    if (blockIdx.x == 0) {
+      a.sh[sn * a.kc + c] = shj == kRaw ? kRaw : shj + q.o;
+      a.mx[sr * a.kc + c] = mj >> 4;  // start of the next vector's maximum
+    }
+  }
+  __syncthreads();
+  if ((int32_t)mine >= a.per_pass || group >= a.groups) return;
+  const bool raw = a.sh[sj * a.kc + c0] == kRaw;
+  const ColumnScale *sc = scale + (slot - mine * a.tile) * CPL;
+  bool plain = true;
+  int32_t big[CPL];
+#pragma unroll
+  for (int c = 0; c < CPL; ++c) {
+    plain = plain && sc[c].o == 0 && (MODE == MODE_FIRST || sc[c].wsh == 0);
+    big[c] = 0;
+  }
+  const int64_t ldb = a.ld * 8;
+  const uint32_t stride = (uint32_t)(3 * ldb);
+  const char *xl = reinterpret_cast<const char *>(a.X + c0);
+  const bool with_y = MODE != MODE_STEP || a.Y != nullptr;
+  for (int32_t atom = first + (int32_t)mine; atom < last; atom += a.per_pass) {
+    if (raw) {
+      raw_step<CPL, MODE, FULL>(a, atom, c0);
+      continue;
+    }
+    int64_t accH[3][CPL], accM[3][CPL];
+#pragma unroll
+    for (int r = 0; r < 3; ++r)
+#pragma unroll
+      for (int c = 0; c < CPL; ++c) {
+        accH[r][c] = 0;
+        accM[r][c] = FULL ? kHalf / 2 : kHalf;  // the final rounding
+      }
+    int32_t p = __ldg(a.rp + atom) - pbase;
+    const int32_t p1 = __ldg(a.rp + atom + 1) - pbase;
+    // the gather of the next block is in flight during the products of one
+    int2 x0[3][CPL], x1[3][CPL];
+    const auto load = [&](int32_t q, int2 (&x)[3][CPL]) {
+      load_atom<CPL>(xl, (uint32_t)sblk[q * kWords + kWords - 1].z, stride, ldb, x);
+    };
+    if (p < p1) load(p, x0);
+    if (!FULL) {
+      load_atom<CPL>(xl, (uint32_t)atom, stride, ldb, x1);
+      const int4 d0 = __ldg(a.dg + 3 * (int64_t)atom), d1 = __ldg(a.dg + 3 * (int64_t)atom + 1),
+                 d2 = __ldg(a.dg + 3 * (int64_t)atom + 2);
+      const int2 xx = make_int2(d0.x, d0.y), xy = make_int2(d0.z, d0.w), xz = make_int2(d1.x, d1.y),
+                 yy = make_int2(d1.z, d1.w), yz = make_int2(d2.x, d2.y), zz = make_int2(d2.z, d2.w);
+      const int2 v[9] = {xx, xy, xz, xy, yy, yz, xz, yz, zz};
+      add_block<CPL>(v, x1, accH, accM);
+    }
+    const int32_t kFold = FULL ? 1 : fold_of(a.info);
+    int32_t until = kFold;
+    for (; p + 1 < p1; p += 2) {
+      load(p + 1, x1);
+      add_neighbour<CPL, FULL>(sblk + p * kWords, x0, accH, accM);
+      if (p + 2 < p1) load(p + 2, x0);
+      add_neighbour<CPL, FULL>(sblk + (p + 1) * kWords, x1, accH, accM);
+      if (--until == 0) {
+        fold<CPL>(accH, accM);
+        until = kFold;
+      }
+    }
+    if (p < p1) add_neighbour<CPL, FULL>(sblk + p * kWords, x0, accH, accM);
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+      const int64_t off = (3 * (int64_t)atom + r) * a.ld + c0;
+      int2 z[CPL], w[CPL], xo[CPL];
+      double y[CPL];
+      if (MODE != MODE_FIRST) load_own<CPL>(a.W + off, w);
+      if (MODE == MODE_FIRST || MODE == MODE_STEP_ACC) load_pairs<CPL>(a.X + off, xo);
+      if (MODE != MODE_FIRST && with_y) load_y<CPL>(a.Y + off, y);
+#pragma unroll
+      for (int c = 0; c < CPL; ++c) {
+        int64_t v = FULL ? (accH[r][c] << 1) + (accM[r][c] >> (kLimb - 1)) : accH[r][c] + (accM[r][c] >> kLimb);
+        if (MODE == MODE_FIRST) {
+          v = shifted(-v, sc[c].o - 1);
+        } else if (plain) {
+          v = -v - join(w[c]);
+        } else {
+          v = shifted(-v - shifted(join(w[c]), sc[c].wsh), sc[c].o);
+        }
+        z[c] = split(v);
+        big[c] = max(big[c], abs(z[c].y));
+      }
+      store_pairs<CPL>(a.Z + off, z);
+      if (with_y) {
+#pragma unroll
+        for (int c = 0; c < CPL; ++c) {
+          int64_t H = mad(a.gb.y, z[c].y, 0), M = mad(a.gb.x, z[c].y, mad(a.gb.y, z[c].x, kHalf));
+          if (MODE == MODE_FIRST || MODE == MODE_STEP_ACC) {
+            if (!plain) xo[c] = split(shifted(join(xo[c]), sc[c].o));
+            H = mad(a.ga.y, xo[c].y, H);
+            M = mad(a.ga.x, xo[c].y, mad(a.ga.y, xo[c].x, M));
+          }
+          const double t = to_double(H + (M >> kLimb));
+          y[c] = MODE == MODE_FIRST ? t * sc[c].ysc : fma(t, sc[c].ysc, y[c]);
+        }
+        store_y<CPL>(a.Y + off, y);
+      }
+    }
+  }
+  if (raw) return;
+#pragma unroll
+  for (int c = 0; c < CPL; ++c) {
+    int32_t *m = a.mx + sn * a.kc + c0 + c;
+    if (big[c] > *reinterpret_cast<volatile int32_t *>(m)) atomicMax(m, big[c]);
+  }
+}
+
+// ---- the operator in fixed point -------------------------------------------------------------
+__device__ __forceinline__ int2 fixed_entry(double v, double unit) { return split(__double2ll_rn(v * unit)); }
+
+// info[0] |= 1 when the operator does not fit; info[1]: ||A||_inf as float bits, rounded up
+__device__ __forceinline__ void note_row(int32_t *info, double row, bool bad) {
+  if (bad || !(row <= 16.0)) atomicOr(info, 1);
+  else atomicMax(info + 1, __float_as_int(__double2float_ru(row * 1.000001)));
+}
+
+// Rank-1 form, unit 2^-60.  With |x| < 2^60 the cross terms of a row's diagonal block and F of its other blocks
+// stay below 2^59 (3 + sum |d| + sum (|u_r| + |u|_1)): info[2], info[3] get the largest such factor for F = 6, 4
+// (below 15.5: 63 bits hold them; F = 2 always does).
+__global__ void k_fixed_r1(int32_t n_atoms, const int32_t *__restrict__ rp1, const int32_t *__restrict__ ci1,
+                           const double *__restrict__ u, const double *__restrict__ dg, int4 *blk, int2 *dgo,
+                           int32_t *info) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n_atoms) return;
+  const double *d = dg + 6 * i;
+  double row[3] = {fabs(d[0]) + fabs(d[1]) + fabs(d[2]), fabs(d[1]) + fabs(d[3]) + fabs(d[4]),
+                   fabs(d[2]) + fabs(d[4]) + fabs(d[5])};
+  bool bad = !(row[0] < 4.0 && row[1] < 4.0 && row[2] < 4.0);
+  for (int t = 0; t < 6; ++t) {
+    bad = bad || !(fabs(d[t]) < 1.99);
+    dgo[6 * i + t] = bad ? make_int2(0, 0) : fixed_entry(-d[t], 0x1p60);
+  }
+  const double drow = fmax(row[0], fmax(row[1], row[2]));
+  double s6[3] = {0, 0, 0}, s4[3] = {0, 0, 0}, m6 = 0.0, m4 = 0.0;
+  const int32_t p0 = rp1[i], p1 = rp1[i + 1];
+  for (int32_t p = p0; p < p1 && !bad; ++p) {
+    const double v[3] = {u[3 * (int64_t)p], u[3 * (int64_t)p + 1], u[3 * (int64_t)p + 2]};
+    const double s = fabs(v[0]) + fabs(v[1]) + fabs(v[2]);
+    if (!(s < 1.9)) {  // u . x has to stay below 2^61 for |x| < 2^60
+      bad = true;
+      break;
+    }
+    const bool new6 = (p - p0) % 6 == 0, new4 = (p - p0) % 4 == 0;
+    for (int r = 0; r < 3; ++r) {
+      row[r] += fabs(v[r]) * s;
+      s6[r] = (new6 ? 0.0 : s6[r]) + fabs(v[r]) + s;
+      s4[r] = (new4 ? 0.0 : s4[r]) + fabs(v[r]) + s;
+      m6 = fmax(m6, s6[r]);
+      m4 = fmax(m4, s4[r]);
+    }
+    const int2 a = fixed_entry(v[0], 0x1p60), b = fixed_entry(v[1], 0x1p60), c = fixed_entry(v[2], 0x1p60);
+    blk[2 * (int64_t)p] = make_int4(a.x, a.y, b.x, b.y);
+    blk[2 * (int64_t)p + 1] = make_int4(c.x, c.y, ci1[p], 0);
+  }
+  if (!bad) {
+    atomicMax(info + 2, __float_as_int((float)(3.0 + drow + m6)));
+    atomicMax(info + 3, __float_as_int((float)(3.0 + drow + m4)));
+  }
+  atomicMax(info + 4, p1 - p0);
+  note_row(info, fmax(row[0], fmax(row[1], row[2])), bad);
+}
+
+// Full blocks, unit 2^-59: the cross terms of two blocks stay below 2^58 sum |a| + 2 x 3 2^59, which 63 bits hold
+// for ||A||_inf <= 16.
+__global__ void k_fixed_full(int32_t n_atoms, const int32_t *__restrict__ rp, const int32_t *__restrict__ ci,
+                             const double *__restrict__ A, int4 *blk, int32_t *info) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n_atoms) return;
+  double row[3] = {0.0, 0.0, 0.0};
+  bool bad = false;
+  for (int32_t p = rp[i]; p < rp[i + 1] && !bad; ++p) {
+    int2 v[10];
+    for (int t = 0; t < 9; ++t) {
+      const double e = A[9 * (int64_t)p + t];
+      bad = bad || !(fabs(e) < 3.9);
+      row[t / 3] += fabs(e);
+      v[t] = bad ? make_int2(0, 0) : fixed_entry(-e, 0x1p59);
+    }
+    v[9] = make_int2(ci[p], 0);
+    for (int t = 0; t < 5; ++t) blk[5 * (int64_t)p + t] = make_int4(v[2 * t].x, v[2 * t].y, v[2 * t + 1].x, v[2 * t + 1].y);
+  }
+  atomicMax(info + 4, rp[i + 1] - rp[i]);
+  note_row(info, fmax(row[0], fmax(row[1], row[2])), bad);
+}
+
+// ---- entry: column maxima, exponents, conversion ---------------------------------------------
+__device__ __forceinline__ uint64_t magnitude(uint64_t bits) { return bits & (~(uint64_t)0 >> 1); }
+
+// Largest |X| bits per column over a slab of rows (patterns of Inf and NaN are the largest): part[slab][c].
+// Row-major: lanes along columns.  Column-major: one block per (slab, column).
+__global__ void __launch_bounds__(256) k_colmax_rm(int64_t n, int32_t k, const uint64_t *__restrict__ X, int64_t ld,
+                                                   int64_t slab, uint64_t *part) {
+  __shared__ uint64_t red[8][33];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int32_t c = blockIdx.y * 32 + lane;
+  const int64_t r0 = (int64_t)blockIdx.x * slab, r1 = min(n, r0 + slab);
+  uint64_t m = 0;
+  if (c < k)
+    for (int64_t i = r0 + warp; i < r1; i += 8) m = max(m, magnitude(X[i * ld + c]));
+  red[warp][lane] = m;
+  __syncthreads();
+  if (warp == 0 && c < k) {
+    for (int w = 1; w < 8; ++w) m = max(m, red[w][lane]);
+    part[(int64_t)blockIdx.x * k + c] = m;
+  }
+}
+__global__ void __launch_bounds__(256) k_colmax_cm(int64_t n, int32_t k, const uint64_t *__restrict__ X, int64_t ld,
+                                                   int64_t slab, uint64_t *part) {
+  __shared__ uint64_t red[8];
+  const int64_t r0 = (int64_t)blockIdx.x * slab, r1 = min(n, r0 + slab);
+  for (int32_t c = blockIdx.y; c < k; c += gridDim.y) {
+    const uint64_t *x = X + (int64_t)c * ld;
+    uint64_t m = 0;
+    for (int64_t i = r0 + threadIdx.x; i < r1; i += 256) m = max(m, magnitude(x[i]));
+    for (int d = 16; d > 0; d >>= 1) m = max(m, (uint64_t)__shfl_xor_sync(0xffffffffu, (unsigned long long)m, d));
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      for (int w = 1; w < 8; ++w) m = max(m, red[w]);
+      part[(int64_t)blockIdx.x * k + c] = m;
+    }
+    __syncthreads();
+  }
+}
+
+// exponent and bound of t_0 per column; cpl adjacent columns are kept in FP64 together
+__global__ void k_fixed_plan(int32_t k, int32_t parts, const uint64_t *__restrict__ part, int32_t cpl,
+                             const int32_t *__restrict__ info, int64_t kc, int32_t *sh, int32_t *mx) {
+  const int64_t c0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * cpl;
+  if (c0 >= kc) return;
+  int32_t s0[2] = {0, 0}, m0[2] = {0, 0};
+  bool raw = false;
+  for (int t = 0; t < cpl; ++t) {
+    const int64_t c = c0 + t;
+    if (c >= k) continue;
+    uint64_t m = 0;
+    for (int32_t q = 0; q < parts; ++q) m = max(m, part[(int64_t)q * k + c]);
+    if (m == 0) continue;
+    const double v = __longlong_as_double((long long)m);
+    if (!(v >= 0x1p-900 && v <= 0x1p900)) {
+      raw = true;
+      continue;
+    }
+    const float g = norm_of(info);
+    s0[t] = top_of(g) - 1 - ilogb(v * ((double)g + 1.0) * 1.0001);
+    m0[t] = (int32_t)ldexp(v, s0[t] - kLimb) + 1;
+  }
+  for (int t = 0; t < cpl; ++t) {
+    sh[c0 + t] = raw ? kRaw : s0[t];
+    mx[c0 + t] = m0[t];
+    mx[kc + c0 + t] = m0[t] >> 4;
+  }
+}
+
+// x 2^s rounded to nearest, from the bits of x (no FP64 instructions); |x| 2^s < 2^60
+__device__ __forceinline__ int2 to_fixed(uint64_t bits, int32_t s) {
+  const int e = (int)(bits >> 52) & 0x7ff;
+  uint64_t m = bits & 0xfffffffffffffull;
+  if (e) m |= 1ull << 52;
+  int64_t v = shifted((int64_t)m, (e ? e : 1) - 1075 + s);
+  return split((int64_t)bits < 0 ? -v : v);
+}
+__device__ __forceinline__ int2 entry(uint64_t bits, int32_t s) {
+  return s == kRaw ? make_int2((int32_t)(uint32_t)bits, (int32_t)(uint32_t)(bits >> 32)) : to_fixed(bits, s);
+}
+
+__global__ void __launch_bounds__(256) k_fixed_from_rm(int64_t n, int32_t k, int32_t kp, const uint64_t *__restrict__ X,
+                                                       int64_t ld, const int32_t *__restrict__ sh, int2 *T) {
+  const int64_t t = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  const int64_t i = t / kp;
+  if (i >= n) return;
+  const int32_t c = (int32_t)(t - i * kp);
+  T[i * ld + c] = c < k ? entry(X[i * ld + c], sh[c]) : make_int2(0, 0);
+}
+
+__global__ void __launch_bounds__(256) k_fixed_from_cm(int64_t n, int32_t k, int32_t kp, const uint64_t *__restrict__ C,
+                                                       int64_t ldc, const int32_t *__restrict__ sh, int2 *T, int64_t ld) {
+  __shared__ uint64_t tile[32][33];
+  const int64_t i0 = (int64_t)blockIdx.x * 32;
+  const int32_t cb = blockIdx.y * 32, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  for (int y = ty; y < 32; y += 8) {
+    const int32_t c = cb + y;
+    const int64_t i = i0 + tx;
+    if (c < k && i < n) tile[y][tx] = C[(int64_t)c * ldc + i];
+  }
+  __syncthreads();
+  const int32_t c = cb + tx;
+  if (c >= kp) return;
+  const int32_t s = c < k ? sh[c] : 0;
+  for (int y = ty; y < 32; y += 8) {
+    const int64_t i = i0 + y;
+    if (i < n) T[i * ld + c] = c < k ? entry(tile[tx][y], s) : make_int2(0, 0);
+  }
+}
+
+template <int CPL, bool FULL>
+void launch_step(int mode, const StepArgs &a, dim3 grid, int threads, size_t smem, cudaStream_t s) {
+  if (mode == MODE_FIRST)
+    PFE_LAUNCH k_fixed_step<CPL, MODE_FIRST, FULL><<<grid, threads, smem, s>>>(a);
+  else if (mode == MODE_STEP_ACC)
+    PFE_LAUNCH k_fixed_step<CPL, MODE_STEP_ACC, FULL><<<grid, threads, smem, s>>>(a);
+  else
+    PFE_LAUNCH k_fixed_step<CPL, MODE_STEP, FULL><<<grid, threads, smem, s>>>(a);
+}
+
+int32_t max_parts(int64_t n) { return (int32_t)std::min<int64_t>(64, (n + 511) / 512); }
+
+}  // namespace
+
+// bytes of a block in shared memory, and what a CTA stages at most (a row has to fit)
+size_t fixed_block_bytes(const Bsr<double> &A) { return A.u ? 32 : 80; }
+constexpr size_t kFixedStage = 24576;
+bool fixed_row_fits(const Bsr<double> &A, int32_t max_row) { return max_row * fixed_block_bytes(A) <= kFixedStage; }
+
+size_t fixed_state_bytes(int64_t n, int32_t k) {
+  const int64_t kc = (k + 3) / 4 * 4;
+  return (size_t)(8 * kc) * sizeof(int32_t) + (size_t)max_parts(n) * (size_t)k * sizeof(uint64_t);
+}
+
+void launch_fixed_operator(const Bsr<double> &A, void *blocks, void *diag, int32_t *info, cudaStream_t s) {
+  cudaMemsetAsync(info, 0, kFixedInfo * sizeof(int32_t), s);
+  const unsigned grid = (unsigned)((A.n_atoms + 127) / 128);
+  if (A.u)
+    PFE_LAUNCH k_fixed_r1<<<grid, 128, 0, s>>>(A.n_atoms, A.rp1, A.ci1, A.u, A.dg, static_cast<int4 *>(blocks),
+                                               static_cast<int2 *>(diag), info);
+  else
+    PFE_LAUNCH k_fixed_full<<<grid, 128, 0, s>>>(A.n_atoms, A.rp, A.ci, A.vals, static_cast<int4 *>(blocks), info);
+}
+
+bool fixed_coefficients_ok(const double *coef, int32_t m) {
+  double g = 0.0;
+  for (int32_t j = 0; j <= m; ++j) g = std::fmax(g, std::fabs(coef[j]));
+  return m >= 1 && g < 0x1p60;
+}
+
+void launch_fixed_filter(const Bsr<double> &A, const FixedOp &op, const double *coef, int32_t m, int32_t k, int64_t ld,
+                         const double *X, int64_t ldx, bool colmajor, double *Y, double *b0, double *b1, void *state,
+                         cudaStream_t s) {
+  const int64_t n = 3 * (int64_t)A.n_atoms, kc = (k + 3) / 4 * 4;
+  int32_t *sh = static_cast<int32_t *>(state), *mx = sh + 4 * kc;
+  uint64_t *part = reinterpret_cast<uint64_t *>(mx + 4 * kc);
+  auto al16 = [](const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
+  // Two columns a lane (16-byte gathers) once the lanes fill the GPU a few times over; before that one, for more
+  // lanes (N = 1,000, k = 16: 9.0 us a step with one, 12.0 with two; N = 5,003, k = 33: 19.8 and 20.7;
+  // N = 99,900, k = 64: 334 and 303).
+  const bool wide = k > 1 && ld % 2 == 0 && al16(Y) && al16(b0) && al16(b1);
+  const int cpl = wide && (int64_t)A.n_atoms * k >= 200000 ? 2 : 1;
+  const int32_t npc = (k + cpl - 1) / cpl, kp = npc * cpl;
+  // exponents of t_0 and its conversion into b1
+  const int32_t parts = max_parts(n);
+  const int64_t slab = (n + parts - 1) / parts;
+  const uint64_t *xb = reinterpret_cast<const uint64_t *>(X);
+  int2 *t0 = reinterpret_cast<int2 *>(b1), *t1 = reinterpret_cast<int2 *>(b0);
+  if (colmajor)
+    PFE_LAUNCH k_colmax_cm<<<dim3(parts, std::min(k, 65535)), 256, 0, s>>>(n, k, xb, ldx, slab, part);
+  else
+    PFE_LAUNCH k_colmax_rm<<<dim3(parts, (k + 31) / 32), 256, 0, s>>>(n, k, xb, ldx, slab, part);
+  PFE_LAUNCH k_fixed_plan<<<(unsigned)((kc / cpl + 127) / 128), 128, 0, s>>>(k, parts, part, cpl, op.info, kc, sh, mx);
+  if (colmajor)
+    PFE_LAUNCH k_fixed_from_cm<<<dim3((unsigned)((n + 31) / 32), (kp + 31) / 32), 256, 0, s>>>(n, k, kp, xb, ldx, sh, t0, ld);
+  else
+    PFE_LAUNCH k_fixed_from_rm<<<(unsigned)((n * kp + 255) / 256), 256, 0, s>>>(n, k, kp, xb, ldx, sh, t0);
+  auto fixed = [](double v, int ge) {  // v 2^(59 - ge), split; |v| <= 2^ge
+    const int64_t t = std::llrint(std::ldexp(v, 2 * kLimb - 1 - ge)) + kHalf;
+    return make_int2((int32_t)(t & kMask) - kHalf, (int32_t)(t >> kLimb));
+  };
+  StepArgs a{};
+  a.n_atoms = A.n_atoms;
+  a.ld = ld;
+  a.rp = A.u ? A.rp1 : A.rp;
+  a.blk = static_cast<const int4 *>(op.blocks);
+  a.dg = static_cast<const int4 *>(op.diag);
+  a.u64 = A.u ? A.u : A.vals;
+  a.d64 = A.dg;
+  a.ci64 = A.u ? A.ci1 : A.ci;
+  a.info = op.info;
+  a.sh = sh;
+  a.mx = mx;
+  a.kc = kc;
+  // CTA shape: the fewest column tiles, evenly wide; as many atoms at a time as 256 lanes hold; up to four passes
+  // while every SM keeps its three CTAs (N = 99,900, k = 64: 318 us a step with one pass, 303 with four, 302 with
+  // eight; N = 5,003, k = 33: 20.7 with one, 24.9 with four).
+  const int tiles = (npc + 255) / 256;
+  a.groups = npc;
+  a.tile = (npc + tiles - 1) / tiles;
+  a.per_pass = 256 / a.tile;
+  a.magic = (65536 + a.tile - 1) / a.tile;
+  const size_t row_bytes = (size_t)op.max_row * fixed_block_bytes(A);
+  while (a.per_pass > 1 && a.per_pass * row_bytes > kFixedStage) --a.per_pass;
+  const int threads = (a.per_pass * a.tile + 31) / 32 * 32;
+  const int64_t ctas = ((int64_t)A.n_atoms + a.per_pass - 1) / a.per_pass * tiles;
+  a.passes = (int32_t)std::min<int64_t>(4, std::max<int64_t>(1, ctas / (3 * 152)));
+  while (a.passes > 1 && a.per_pass * a.passes * row_bytes > kFixedStage) --a.passes;
+  const int per_cta = a.per_pass * a.passes;
+  const size_t smem = (size_t)a.tile * cpl * sizeof(ColumnScale) + per_cta * row_bytes;
+  const dim3 grid((unsigned)((A.n_atoms + per_cta - 1) / per_cta), (unsigned)tiles);
+  for (int32_t j = 0; j < m; ++j) {
+    // y takes two terms every other step, as in the FP64 filter
+    const bool even = (j % 2) == 0, last = j == m - 1;
+    const int mode = j == 0 ? MODE_FIRST : even ? MODE_STEP_ACC : MODE_STEP;
+    a.j = j;
+    a.X = even ? t0 : t1;
+    a.W = a.Z = even ? t1 : t0;
+    a.Y = (even || last) ? Y : nullptr;
+    const double g = std::fmax(even ? std::fabs(coef[j]) : 0.0, std::fabs(coef[j + 1]));
+    a.ge = g > 0.0 ? std::ilogb(g) + 1 : 0;  // the pair's own exponent: a small pair keeps its relative accuracy
+    a.ga = even ? fixed(coef[j], a.ge) : make_int2(0, 0);
+    a.gb = fixed(coef[j + 1], a.ge);
+    a.g0 = coef[j];
+    a.g1 = coef[j + 1];
+    if (A.u) {
+      if (cpl == 2) launch_step<2, false>(mode, a, grid, threads, smem, s);
+      else launch_step<1, false>(mode, a, grid, threads, smem, s);
+    } else {
+      if (cpl == 2) launch_step<2, true>(mode, a, grid, threads, smem, s);
+      else launch_step<1, true>(mode, a, grid, threads, smem, s);
+    }
+  }
+}
+
+}  // namespace pfe

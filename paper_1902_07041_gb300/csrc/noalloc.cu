@@ -63,6 +63,17 @@ extern "C" pfe_status pfe_filter_apply_noalloc(pfe_ctx *ctx, int32_t m, const do
     cudaError_t e = cudaStreamSynchronize(ctx->stream);
     if (e != cudaSuccess) return pfe_fail(ctx, PFE_E_CUDA, std::string("cudaStreamSynchronize: ") + cudaGetErrorString(e));
   }
+  // The fixed-point filter when its operator is built; its per-column state takes the place of the row-major
+  // copy of X, which it does not need.
+  const FixedOp op = solver_fixed_op(ctx, coeffs, m);
+  if (op.blocks && fixed_state_bytes(n, k) <= (size_t)(n * ld) * sizeof(double)) {
+    launch_fixed_filter(solver_bsr_Hs64(ctx), op, coeffs, m, k, ld, X, ldx, true, Yr, b0, b1, Xr, s);
+    launch_rowmajor_to_colmajor<double>(n, k, Yr, ld, Y, ldy, s);
+    cudaError_t fe = cudaGetLastError();
+    if (fe != cudaSuccess)
+      return pfe_fail(ctx, PFE_E_CUDA, std::string("filter_apply_noalloc: ") + cudaGetErrorString(fe));
+    return PFE_OK;
+  }
   // The array keeps the previous call's contents.  Columns are independent, so only the padding
   // columns k .. ld-1 of the four blocks (read by the vector lanes, never copied out) are cleared.
   if (ld > k) {

@@ -154,6 +154,26 @@ void launch_zero(T *p, int64_t count, cudaStream_t s);
 // *out = max |G - I| over a k x k matrix (device scalar)
 void launch_max_dev_identity(int32_t k, const double *G, double *out, cudaStream_t s);
 
+// The FP64 filter in 64-bit fixed point (fixed_step.cu).  FixedOp: the filter operator split into limbs
+// (rank-1: two int4 per off-diagonal block and six int2 per atom; full: five int4 per block), info on the device
+// (info[0] != 0 when it does not fit, then bounds; see fixed_step.cu) and the longest row's block count
+constexpr int kFixedInfo = 8;
+struct FixedOp {
+  const void *blocks = nullptr, *diag = nullptr;
+  int32_t *info = nullptr;
+  int32_t max_row = 0;
+};
+size_t fixed_state_bytes(int64_t n, int32_t k);  // the per-column state of one filter call
+void launch_fixed_operator(const Bsr<double> &A, void *blocks, void *diag, int32_t *info, cudaStream_t s);
+bool fixed_row_fits(const Bsr<double> &A, int32_t max_row);
+bool fixed_coefficients_ok(const double *coef, int32_t m);
+// Y (row-major n x ld, doubles) = sum_j coef[j] T_j X; X row-major (ldx == ld) or column-major; b0, b1: n x ld
+// words of 8 bytes, state: fixed_state_bytes(n, k)
+void launch_fixed_filter(const Bsr<double> &A, const FixedOp &op, const double *coef, int32_t m, int32_t k, int64_t ld,
+                         const double *X, int64_t ldx, bool colmajor, double *Y, double *b0, double *b1, void *state,
+                         cudaStream_t s);
+constexpr int kFixedShape = 12;  // its number among the kernel shapes in pfe_stats
+
 // Batched filter: one persistent launch per Chebyshev step over every sample's work items.
 // One descriptor per sample (device-resident, refreshed before every graph replay).
 struct BatchDesc {
@@ -283,6 +303,11 @@ struct pfe_ctx {
   pfe::DBuf r1_rp, r1_ci, r1_u64, r1_dg64, r1_u32, r1_dg32, r1_flag;
   int r1_state = -1;
   bool r1_32 = false;
+  // the filter operator in fixed point (fixed_step.cu), built by the first FP64 filter call on it:
+  // fx_kind 0 = not built, 1 = rank-1 form, 2 = full blocks, -1/-2 = that form does not fit
+  pfe::DBuf fx_blocks, fx_diag, fx_info, w_fx;
+  int fx_kind = 0;
+  int32_t fx_max_row = 0;
   pfe::DBuf t_ptr, t_atoms, t_slot1, t_self;  // tiles of the staged FP32 step (built with the FP32 form)
   int32_t t_umax = 0;
 
@@ -365,6 +390,8 @@ pfe_status solver_filter64(pfe_ctx *ctx, int32_t k, int64_t ld, const double *X,
 // when built), on stream s; tune = false runs the already tuned kernel shape without timing candidates
 pfe_status solver_filter64_rows(pfe_ctx *ctx, const double *coef, int32_t m, int32_t k, int64_t ld, const double *X,
                                 double *Y, double *b0, double *b1, cudaStream_t s, bool tune);
+// the fixed-point operator when it is built and serves this filter (no allocation, no wait); blocks null otherwise
+FixedOp solver_fixed_op(const pfe_ctx *ctx, const double *coef, int32_t m);
 double solver_now();
 pfe_status solver_ensure_lmax(pfe_ctx *ctx);
 Bsr<double> solver_bsr_H(const pfe_ctx *ctx);     // H

@@ -121,6 +121,44 @@ pfe_status run_filter(pfe_ctx *ctx, const Bsr<T> &A, const double *coef, int32_t
   return check_launch(ctx, "filter step");
 }
 
+// The fixed-point form of the FP64 filter operator A, built once per operator (allocates, waits for its check).
+pfe_status ensure_fixed(pfe_ctx *ctx, const Bsr<double> &A) {
+  const int kind = A.u ? 1 : 2;
+  if (std::abs(ctx->fx_kind) == kind) return PFE_OK;
+  const size_t noff = (size_t)(ctx->nnzb - ctx->N), n1 = std::max<size_t>(noff, 1);
+  RESERVE(int32_t, blocks, ctx->fx_blocks, A.u ? 8 * n1 : 20 * (size_t)ctx->nnzb);
+  RESERVE(int32_t, diag, ctx->fx_diag, A.u ? 12 * (size_t)ctx->N : 4);
+  RESERVE(int32_t, info, ctx->fx_info, kFixedInfo);
+  launch_fixed_operator(A, blocks, diag, info, ctx->stream);
+  PFE_TRY(check_launch(ctx, "fixed-point filter operator"));
+  int32_t h[kFixedInfo] = {1};
+  PFE_CUDA_TRY(ctx, cudaMemcpyAsync(h, info, sizeof(h), cudaMemcpyDeviceToHost, ctx->stream));
+  PFE_CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));
+  ctx->fx_kind = h[0] || !fixed_row_fits(A, h[4]) ? -kind : kind;
+  ctx->fx_max_row = h[4];
+  return PFE_OK;
+}
+
+// The FP64 filter: in fixed point (fixed_step.cu) unless a kernel shape is forced, the operator or the
+// coefficients do not fit, or the degree is 0.  X row-major (ldx == ld) or, with Xr != null, column-major; Xr is
+// then the row-major copy that the FP64 kernels take.
+pfe_status run_filter64(pfe_ctx *ctx, const Bsr<double> &A, const double *coef, int32_t m, int32_t k, int64_t ld,
+                        const double *X, int64_t ldx, double *Xr, double *Y, double *b0, double *b1, cudaStream_t s) {
+  if (k <= 0) return PFE_OK;
+  if (step_variant(0) < 0 && fixed_coefficients_ok(coef, m)) {
+    PFE_TRY(ensure_fixed(ctx, A));
+    const FixedOp op = solver_fixed_op(ctx, coef, m);
+    if (op.blocks) {
+      RESERVE(char, state, ctx->w_fx, fixed_state_bytes(ctx->n, k));
+      launch_fixed_filter(A, op, coef, m, k, ld, X, ldx, Xr != nullptr, Y, b0, b1, state, s);
+      note_step_variant(0, kFixedShape);
+      return check_launch(ctx, "fixed-point filter");
+    }
+  }
+  if (Xr) launch_colmajor_to_rowmajor<double>(ctx->n, k, X, ldx, Xr, ld, s);
+  return run_filter<double>(ctx, A, coef, m, k, ld, Xr ? Xr : X, Y, b0, b1, s);
+}
+
 // ---------------------------------------------------------------- set-up helpers
 pfe_status ensure_lmax(pfe_ctx *ctx);
 
@@ -246,6 +284,7 @@ pfe_status ensure_hs(pfe_ctx *ctx, bool need32) {
     RESERVE(float, p32, ctx->Hs32, (size_t)9 * ctx->nnzb);
     h32 = p32;
   }
+  ctx->fx_kind = 0;
   launch_filter_matrix(ctx->N, ctx->rp.as<int32_t>(), ctx->ci.as<int32_t>(), ctx->H.as<double>(), 2.0 / ctx->td, ctx->tc,
                        h64, h32, ctx->stream);
   PFE_TRY(check_launch(ctx, "filter matrix"));
@@ -372,7 +411,7 @@ pfe_status estimate_count(pfe_ctx *ctx, double lo, double hi, double *out) {
   chi_coefficients(xi, eta, deg, gam);
   damping_factors(ctx->p_count_damping, deg, g);
   for (int32_t j = 0; j <= deg; ++j) gam[j] *= g[j];
-  PFE_TRY(run_filter<double>(ctx, bsr_Hs64(ctx), gam.data(), deg, M, ld, V, Y, b0, b1, s));
+  PFE_TRY(run_filter64(ctx, bsr_Hs64(ctx), gam.data(), deg, M, ld, V, ld, nullptr, Y, b0, b1, s));
   launch_col_dots<double>(n, M, V, ld, Y, ld, dots, red, s);
   std::vector<double> vy(M);
   PFE_CUDA_TRY(ctx, cudaMemcpyAsync(vy.data(), dots, sizeof(double) * M, cudaMemcpyDeviceToHost, s));
@@ -724,7 +763,7 @@ pfe_status solve_filter(pfe_ctx *ctx) {
   if (k64 > 0) {
     st.f_launch += m1;
     st.f_cols64 += (int64_t)k64 * m1;
-    PFE_TRY(run_filter<double>(ctx, bsr_Hs64(ctx), ctx->coef.data(), ctx->m, k64, ld, st.X, st.Y, st.T0, st.T1, s));
+    PFE_TRY(run_filter64(ctx, bsr_Hs64(ctx), ctx->coef.data(), ctx->m, k64, ld, st.X, ld, nullptr, st.Y, st.T0, st.T1, s));
     ++st.fp64_sweeps;
   }
   if (split) {
@@ -1161,7 +1200,12 @@ pfe_status solver_cholqr2(pfe_ctx *ctx, double *Y, double *tmp, int32_t k, int64
   return cholqr2(ctx, Y, tmp, k, ld, result, shifted);
 }
 pfe_status solver_filter64(pfe_ctx *ctx, int32_t k, int64_t ld, const double *X, double *Y, double *b0, double *b1) {
-  return run_filter<double>(ctx, bsr_Hs64(ctx), ctx->coef.data(), ctx->m, k, ld, X, Y, b0, b1, ctx->stream);
+  return run_filter64(ctx, bsr_Hs64(ctx), ctx->coef.data(), ctx->m, k, ld, X, ld, nullptr, Y, b0, b1, ctx->stream);
+}
+FixedOp solver_fixed_op(const pfe_ctx *ctx, const double *coef, int32_t m) {
+  const bool r1 = ctx->p_rank1 && ctx->r1_state == 1;
+  if (ctx->fx_kind != (r1 ? 1 : 2) || step_variant(0) >= 0 || !fixed_coefficients_ok(coef, m)) return FixedOp{};
+  return FixedOp{ctx->fx_blocks.p, ctx->fx_diag.p, ctx->fx_info.as<int32_t>(), ctx->fx_max_row};
 }
 pfe_status solver_filter64_rows(pfe_ctx *ctx, const double *coef, int32_t m, int32_t k, int64_t ld, const double *X,
                                 double *Y, double *b0, double *b1, cudaStream_t s, bool tune) {
@@ -1363,7 +1407,8 @@ void pfe_destroy(pfe_ctx *ctx) {
                   &ctx->w_bks[0], &ctx->w_bks[1], &ctx->w_bks[2], &ctx->w_bks[3], &ctx->w_bks[4],
                   &ctx->r1_rp, &ctx->r1_ci, &ctx->r1_u64, &ctx->r1_dg64, &ctx->r1_u32, &ctx->r1_dg32,
                   &ctx->r1_flag, &ctx->w_slice[0], &ctx->w_slice[1], &ctx->w_f32e, &ctx->w_defect, &ctx->w_tau,
-                  &ctx->t_ptr, &ctx->t_atoms, &ctx->t_slot1, &ctx->t_self};
+                  &ctx->t_ptr, &ctx->t_atoms, &ctx->t_slot1, &ctx->t_self, &ctx->fx_blocks, &ctx->fx_diag,
+                  &ctx->fx_info, &ctx->w_fx};
   for (DBuf *b : bufs) dbuf_free(*b);
   for (int e = 0; e < 4; ++e)
     if (ctx->solve.ev[e]) cudaEventDestroy(ctx->solve.ev[e]);
@@ -1734,8 +1779,7 @@ pfe_status pfe_filter_apply(pfe_ctx *ctx, int32_t m, const double *coeffs, int32
     RESERVE(double, Yr, ctx->w_Y, big);
     RESERVE(double, b0, ctx->w_T0, big);
     RESERVE(double, b1, ctx->w_T1, big);
-    launch_colmajor_to_rowmajor<double>(n, k, static_cast<const double *>(X), ldx, Xr, ld, s);
-    PFE_TRY(run_filter<double>(ctx, bsr_Hs64(ctx), cf, m, k, ld, Xr, Yr, b0, b1, s));
+    PFE_TRY(run_filter64(ctx, bsr_Hs64(ctx), cf, m, k, ld, static_cast<const double *>(X), ldx, Xr, Yr, b0, b1, s));
     launch_rowmajor_to_colmajor<double>(n, k, Yr, ld, static_cast<double *>(Y), ldy, s);
   } else {
     RESERVE(float, Xr, ctx->w_f32a, big);
