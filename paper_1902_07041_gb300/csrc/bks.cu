@@ -54,8 +54,8 @@ void project(pfe_ctx *ctx, const double *V, int64_t ldv, int32_t nv, double *W, 
              double *gw, int passes) {
   if (nv <= 0 || k <= 0) return;
   for (int pass = 0; pass < passes; ++pass) {
-    launch_gram(ctx->n, nv, k, V, ldv, W, ldw, 1.0, 0.0, h, nv, false, gw, ctx->stream);
-    launch_update(ctx->n, k, nv, V, ldv, h, nv, -1.0, 1.0, W, ldw, ctx->stream);
+    launch_gram(ctx->n, nv, k, V, ldv, W, ldw, 1.0, 0.0, h, nv, false, gw, ctx->stream, &ctx->w_digits);
+    launch_update(ctx->n, k, nv, V, ldv, h, nv, -1.0, 1.0, W, ldw, ctx->stream, false, &ctx->w_digits);
   }
 }
 
@@ -177,15 +177,15 @@ pfe_status bks_solve(pfe_ctx *ctx, int32_t *n_found) {
       launch_axpby<double>(n, bs, 1.0, Yb, ldb, 0.0, Wb, ldb, s);
       // first pass: T[0:nv+bs, nv:nv+bs] = V^T Op V_j, then W -= V T[0:nv+bs, nv:nv+bs]
       double *Tcol = Tm + (size_t)nv * ldT;
-      launch_gram(n, nv + bs, bs, V, ldv, Wb, ldb, 1.0, 0.0, Tcol, ldT, false, gw, s);
-      launch_update(n, bs, nv + bs, V, ldv, Tcol, ldT, -1.0, 1.0, Wb, ldb, s);
+      launch_gram(n, nv + bs, bs, V, ldv, Wb, ldb, 1.0, 0.0, Tcol, ldT, false, gw, s, &ctx->w_digits);
+      launch_update(n, bs, nv + bs, V, ldv, Tcol, ldT, -1.0, 1.0, Wb, ldb, s, false, &ctx->w_digits);
       PFE_TRY(orthonormalise_block(ctx, V, ldv, nv + bs, Wb, T0b, ldb, bs, h, gw, 1));
       launch_axpby<double>(n, bs, 1.0, Wb, ldb, 0.0, V + nv + bs, ldv, s);
       nv += bs;
       timed(t_orth);
     }
     // ---- Ritz pairs of T; B = V_new^T Op V_last (Yb holds Op V_last)
-    launch_gram(n, bs, bs, V + nv, ldv, Yb, ldb, 1.0, 0.0, Bm, bs, false, gw, s);
+    launch_gram(n, bs, bs, V + nv, ldv, Yb, ldb, 1.0, 0.0, Bm, bs, false, gw, s, &ctx->w_digits);
     PFE_CUDA_TRY(ctx, cudaMemcpy2DAsync(A, sizeof(double) * nv, Tm, sizeof(double) * ldT, sizeof(double) * nv, nv,
                                         cudaMemcpyDeviceToDevice, s));
     int lw = 0;
@@ -247,7 +247,7 @@ pfe_status bks_solve(pfe_ctx *ctx, int32_t *n_found) {
       sel_res.clear();
       bool bad = false;
       if (k > 0) {
-        launch_update(n, k, nv, V, ldv, A + (size_t)(nv - k) * nv, nv, 1.0, 0.0, Vn, ldv, s);
+        launch_update(n, k, nv, V, ldv, A + (size_t)(nv - k) * nv, nv, 1.0, 0.0, Vn, ldv, s, false, &ctx->w_digits);
         launch_bsr_step<double>(Hb, MODE_SPMM, k, ldv, Vn, nullptr, HW, nullptr, 1.0, 0.0, 0.0, 0.0, s);
         matvecs += k;
         {
@@ -255,13 +255,13 @@ pfe_status bks_solve(pfe_ctx *ctx, int32_t *n_found) {
           gw = gw2;  // the buffer may have grown
         }
         double *G = Tm;  // T is rebuilt by the restart below if the iteration has to continue
-        launch_gram(n, k, k, Vn, ldv, HW, ldv, 1.0, 0.0, G, k, true, gw, s);  // Yw^T H Yw: symmetric
+        launch_gram(n, k, k, Vn, ldv, HW, ldv, 1.0, 0.0, G, k, true, gw, s, &ctx->w_digits);  // Yw^T H Yw: symmetric
         PFE_SOLVER_TRY(ctx, cusolverDnDsyevd_bufferSize(ctx->solver, CUSOLVER_EIG_MODE_VECTOR, CUBLAS_FILL_MODE_UPPER, k,
                                                         G, k, fin_lam, &lw));
         BKS_RESERVE(double, work2, ctx->w_cs_work, (size_t)std::max(lw, 1));
         PFE_SOLVER_TRY(ctx, cusolverDnDsyevd(ctx->solver, CUSOLVER_EIG_MODE_VECTOR, CUBLAS_FILL_MODE_UPPER, k, G, k,
                                              fin_lam, work2, lw, info));
-        launch_update(n, k, k, Vn, ldv, G, k, 1.0, 0.0, Z, ldv, s);  // U = Yw Q
+        launch_update(n, k, k, Vn, ldv, G, k, 1.0, 0.0, Z, ldv, s, false, &ctx->w_digits);  // U = Yw Q
         launch_bsr_step<double>(Hb, MODE_SPMM, k, ldv, Z, nullptr, HW, nullptr, 1.0, 0.0, 0.0, 0.0, s);
         matvecs += k;
         launch_col_resid2(n, k, HW, Z, ldv, fin_lam, fin_r2, red, s);
@@ -299,7 +299,7 @@ pfe_status bks_solve(pfe_ctx *ctx, int32_t *n_found) {
       break;
     }
     // ---- thick restart: [V S[:, nv-keep:nv] | V[:, nv:nv+bs]] becomes the basis, T = diag(theta_kept)
-    launch_update(n, keep, nv, V, ldv, A + (size_t)(nv - keep) * nv, nv, 1.0, 0.0, Vn, ldv, s);
+    launch_update(n, keep, nv, V, ldv, A + (size_t)(nv - keep) * nv, nv, 1.0, 0.0, Vn, ldv, s, false, &ctx->w_digits);
     launch_axpby<double>(n, bs, 1.0, V + nv, ldv, 0.0, Wb, ldb, s);
     std::swap(V, Vn);
     PFE_TRY(orthonormalise_block(ctx, V, ldv, keep, Wb, T0b, ldb, bs, h, gw, 2));

@@ -218,11 +218,20 @@ void launch_defect_combine(int64_t n, int32_t act, const double *X, int64_t ld, 
 int32_t gram_splits(int64_t K, int32_t m, int32_t nn, bool sym);
 size_t gram_work(int64_t K, int32_t m, int32_t nn, bool sym);
 void launch_gram(int64_t K, int32_t m, int32_t nn, const double *A, int64_t lda, const double *B, int64_t ldb,
-                 double alpha, double beta, double *C, int64_t ldc, bool sym, double *work, cudaStream_t s);
+                 double alpha, double beta, double *C, int64_t ldc, bool sym, double *work, cudaStream_t s,
+                 DBuf *digits = nullptr);
 // C (M x N row-major, ldc) = alpha A (M x K row-major, lda) Bc (K x N column-major, ldb) + beta C
 void launch_update(int64_t M, int32_t N, int32_t K, const double *A, int64_t lda, const double *Bc, int64_t ldb,
                    double alpha, double beta, double *C, int64_t ldc, cudaStream_t s,
-                   bool upper = false);
+                   bool upper = false, DBuf *digits = nullptr);
+// With a buffer `digits` (grown as needed; without room the products stay on the FP64 path) large products run on the
+// BF16 tensor cores by exact digits (digit_gemm.cu).
+size_t digit_gram_bytes(int64_t K, int32_t m, int32_t nn, bool same);
+void launch_gram_digits(int64_t K, int32_t m, int32_t nn, const double *A, int64_t lda, const double *B, int64_t ldb,
+                        double alpha, double beta, double *C, int64_t ldc, bool sym, void *work, cudaStream_t s);
+size_t digit_update_bytes(int64_t M, int32_t N, int32_t K);
+void launch_update_digits(int64_t M, int32_t N, int32_t K, const double *A, int64_t lda, const double *Bc, int64_t ldb,
+                          double alpha, double beta, double *C, int64_t ldc, bool upper, void *work, cudaStream_t s);
 
 // --------------------------------------------------------------------------------------
 // Host math of the filter (App. A, Sec. 2.3, eq. (thresh)); independent of the oracle
@@ -367,7 +376,7 @@ struct pfe_ctx {
 
   // workspaces
   pfe::DBuf w_X, w_Y, w_W, w_T0, w_T1, w_T2, w_small, w_small2, w_red, w_idx, w_cs_work, w_info, w_f32a, w_f32b,
-      w_f32c, w_f32d, w_ckpt, w_rr, w_gram, w_bks[5], w_slice[2], w_f32e, w_defect, w_tau;
+      w_f32c, w_f32d, w_ckpt, w_rr, w_gram, w_digits, w_bks[5], w_slice[2], w_f32e, w_defect, w_tau;
   int64_t launch_base = 0;  // process-wide launch counter when the context was created
   SolveState solve;
   pfe::DBuf dcoef;            // filter coefficients on the device (batched solves)

@@ -255,7 +255,7 @@ extern "C" pfe_status pfe_solve_sliced(pfe_ctx *ctx, int32_t nedges, const doubl
     PFE_CUDA_TRY(ctx, cudaMemcpyAsync(didx, cols.data(), sizeof(int32_t) * z, cudaMemcpyHostToDevice, s));
     launch_gather_cols(n, z, acc->as<double>(), ldacc, W, ldz, didx, s);
     // W^T W = S diag(ev) S^T; keep the directions with ev > 1/2, scaled by ev^{-1/2}
-    launch_gram(n, z, z, W, ldz, W, ldz, 1.0, 0.0, G, z, false, gw, s);
+    launch_gram(n, z, z, W, ldz, W, ldz, 1.0, 0.0, G, z, false, gw, s, &ctx->w_digits);
     int lw = 0;
     PFE_SOLVER_TRY(ctx, cusolverDnDsyevd_bufferSize(ctx->solver, CUSOLVER_EIG_MODE_VECTOR, CUBLAS_FILL_MODE_UPPER, z, G,
                                                     z, ev, &lw));
@@ -277,17 +277,17 @@ extern "C" pfe_status pfe_solve_sliced(pfe_ctx *ctx, int32_t nedges, const doubl
         ++r;
       }
     PFE_CUDA_TRY(ctx, cudaMemcpyAsync(Sv, hB.data(), sizeof(double) * hB.size(), cudaMemcpyHostToDevice, s));
-    launch_update(n, r, z, W, ldz, Sv, z, 1.0, 0.0, Q, ldz, s);  // orthonormal basis of the joint span
+    launch_update(n, r, z, W, ldz, Sv, z, 1.0, 0.0, Q, ldz, s, false, &ctx->w_digits);  // orthonormal basis of the joint span
     PFE_CUDA_TRY(ctx, cudaStreamSynchronize(s));                  // hB must outlive its copy
     // Rayleigh-Ritz with H on Q
     launch_bsr_step<double>(Hb, MODE_SPMM, r, ldz, Q, nullptr, HQ, nullptr, 1.0, 0.0, 0.0, 0.0, s);
-    launch_gram(n, r, r, Q, ldz, HQ, ldz, 1.0, 0.0, G, r, false, gw, s);
+    launch_gram(n, r, r, Q, ldz, HQ, ldz, 1.0, 0.0, G, r, false, gw, s, &ctx->w_digits);
     PFE_SOLVER_TRY(ctx, cusolverDnDsyevd_bufferSize(ctx->solver, CUSOLVER_EIG_MODE_VECTOR, CUBLAS_FILL_MODE_UPPER, r, G,
                                                     r, ev, &lw));
     SL_RESERVE(double, work2, ctx->w_cs_work, (size_t)std::max(lw, 1));
     PFE_SOLVER_TRY(ctx, cusolverDnDsyevd(ctx->solver, CUSOLVER_EIG_MODE_VECTOR, CUBLAS_FILL_MODE_UPPER, r, G, r, ev,
                                          work2, lw, info));
-    launch_update(n, r, r, Q, ldz, G, r, 1.0, 0.0, W, ldz, s);  // Ritz vectors U = Q Y (into W)
+    launch_update(n, r, r, Q, ldz, G, r, 1.0, 0.0, W, ldz, s, false, &ctx->w_digits);  // Ritz vectors U = Q Y (into W)
     launch_bsr_step<double>(Hb, MODE_SPMM, r, ldz, W, nullptr, HQ, nullptr, 1.0, 0.0, 0.0, 0.0, s);
     launch_col_resid2(n, r, HQ, W, ldz, ev, r2, red, s);
     std::vector<double> lam(r), rr(r);

@@ -443,7 +443,7 @@ pfe_status window_estimate(pfe_ctx *ctx, double *out) {
 // G = Y^T Y by the DMMA Gram kernel (upper tiles, mirrored)
 pfe_status gram_sym(pfe_ctx *ctx, const double *Y, int32_t k, int64_t ld, double *G) {
   RESERVE(double, gw, ctx->w_gram, gram_work(ctx->n, k, k, true));
-  launch_gram(ctx->n, k, k, Y, ld, Y, ld, 1.0, 0.0, G, k, true, gw, ctx->stream);
+  launch_gram(ctx->n, k, k, Y, ld, Y, ld, 1.0, 0.0, G, k, true, gw, ctx->stream, &ctx->w_digits);
   return check_launch(ctx, "Gram");
 }
 
@@ -523,7 +523,7 @@ pfe_status cholqr2(pfe_ctx *ctx, double *Y, double *tmp, int32_t k, int64_t ld, 
     bool shifted = false;
     PFE_TRY(chol_factor(ctx, G, Rinv, k, &shifted));
     any_shift = any_shift || shifted;
-    launch_update(ctx->n, k, k, src, ld, Rinv, k, 1.0, 0.0, dst, ld, s, true);  // R^{-1} is upper triangular
+    launch_update(ctx->n, k, k, src, ld, Rinv, k, 1.0, 0.0, dst, ld, s, true, &ctx->w_digits);  // R^{-1} is upper triangular
     PFE_TRY(check_launch(ctx, "CholeskyQR update"));
     *result = dst;
     std::swap(src, dst);
@@ -540,8 +540,8 @@ pfe_status project_out(pfe_ctx *ctx, const double *L, int32_t nl, double *Y, int
   const int64_t n = ctx->n;
   RESERVE(double, h, ctx->w_small2, (size_t)nl * k);
   RESERVE(double, gw, ctx->w_gram, gram_work(n, nl, k, false));
-  launch_gram(n, nl, k, L, ld, Y, ld, 1.0, 0.0, h, nl, false, gw, ctx->stream);
-  launch_update(n, k, nl, L, ld, h, nl, -1.0, 1.0, Y, ld, ctx->stream);
+  launch_gram(n, nl, k, L, ld, Y, ld, 1.0, 0.0, h, nl, false, gw, ctx->stream, &ctx->w_digits);
+  launch_update(n, k, nl, L, ld, h, nl, -1.0, 1.0, Y, ld, ctx->stream, false, &ctx->w_digits);
   return check_launch(ctx, "projection");
 }
 
@@ -800,7 +800,7 @@ pfe_status solve_after_filter(pfe_ctx *ctx) {
   {
     // A = X^T H X is symmetric: only the upper tiles are computed (half the flops), then mirrored
     RESERVE(double, gw, ctx->w_gram, gram_work(n, act, act, true));
-    launch_gram(n, act, act, st.X, ld, st.W, ld, 1.0, 0.0, st.A, act, true, gw, s);
+    launch_gram(n, act, act, st.X, ld, st.W, ld, 1.0, 0.0, st.A, act, true, gw, s, &ctx->w_digits);
   }
   int lw = 0;
   if (G1) {
@@ -817,7 +817,7 @@ pfe_status solve_after_filter(pfe_ctx *ctx) {
     PFE_SOLVER_TRY(ctx, cusolverDnDsyevd(ctx->solver, CUSOLVER_EIG_MODE_VECTOR, CUBLAS_FILL_MODE_UPPER, act, st.A, act,
                                          st.evals, work, lw, st.info));
   }
-  launch_update(n, act, act, st.X, ld, st.A, act, 1.0, 0.0, st.Y, ld, s);
+  launch_update(n, act, act, st.X, ld, st.A, act, 1.0, 0.0, st.Y, ld, s, false, &ctx->w_digits);
   std::swap(st.X, st.Y);
   // W = H X again on the rotated block: one BSR product instead of the n x q x q update W <- W Q
   launch_bsr_step<double>(bsr_H(ctx), MODE_SPMM, act, ld, st.X, nullptr, st.W, nullptr, 1.0, 0.0, 0.0, 0.0, s);
@@ -1403,7 +1403,7 @@ void pfe_destroy(pfe_ctx *ctx) {
   DBuf *bufs[] = {&ctx->rp, &ctx->ci, &ctx->H, &ctx->mass, &ctx->Hs64, &ctx->Hs32, &ctx->L, &ctx->w_X, &ctx->w_Y,
                   &ctx->w_W, &ctx->w_T0, &ctx->w_T1, &ctx->w_T2, &ctx->w_small, &ctx->w_small2, &ctx->w_red,
                   &ctx->w_idx, &ctx->w_cs_work, &ctx->w_info, &ctx->w_f32a, &ctx->w_f32b, &ctx->w_f32c,
-                  &ctx->w_f32d, &ctx->w_ckpt, &ctx->w_rr, &ctx->w_gram,
+                  &ctx->w_f32d, &ctx->w_ckpt, &ctx->w_rr, &ctx->w_gram, &ctx->w_digits,
                   &ctx->w_bks[0], &ctx->w_bks[1], &ctx->w_bks[2], &ctx->w_bks[3], &ctx->w_bks[4],
                   &ctx->r1_rp, &ctx->r1_ci, &ctx->r1_u64, &ctx->r1_dg64, &ctx->r1_u32, &ctx->r1_dg32,
                   &ctx->r1_flag, &ctx->w_slice[0], &ctx->w_slice[1], &ctx->w_f32e, &ctx->w_defect, &ctx->w_tau,
@@ -1927,7 +1927,7 @@ pfe_status pfe_solve_batch(pfe_ctx **ctxs, int32_t nsamples, int32_t *n_found) {
     // afterwards, one at a time.
     auto work_bufs = [](pfe_ctx *c) {
       return std::vector<DBuf *>{&c->w_X, &c->w_Y, &c->w_W, &c->w_T0, &c->w_T1, &c->w_T2, &c->w_small, &c->w_small2,
-                                 &c->w_red, &c->w_cs_work, &c->w_ckpt, &c->w_rr, &c->w_gram, &c->w_bks[0],
+                                 &c->w_red, &c->w_cs_work, &c->w_ckpt, &c->w_rr, &c->w_gram, &c->w_digits, &c->w_bks[0],
                                  &c->w_bks[1], &c->w_bks[2], &c->w_bks[3], &c->w_bks[4]};
     };
     std::vector<int32_t> order(nsamples);
@@ -1983,7 +1983,7 @@ pfe_status pfe_solve_batch(pfe_ctx **ctxs, int32_t nsamples, int32_t *n_found) {
   // the work buffers of a subspace-iteration solve (the locked vectors L hold the results and stay)
   auto release_si_work = [](pfe_ctx *c) {
     cudaStreamSynchronize(c->stream);
-    for (DBuf *b : {&c->w_X, &c->w_Y, &c->w_W, &c->w_T0, &c->w_T1, &c->w_rr, &c->w_red, &c->w_gram, &c->w_small,
+    for (DBuf *b : {&c->w_X, &c->w_Y, &c->w_W, &c->w_T0, &c->w_T1, &c->w_rr, &c->w_red, &c->w_gram, &c->w_digits, &c->w_small,
                     &c->w_small2, &c->w_cs_work, &c->w_f32a, &c->w_f32b, &c->w_f32c, &c->w_f32d, &c->w_f32e,
                     &c->w_defect, &c->w_tau})
       dbuf_free(*b);

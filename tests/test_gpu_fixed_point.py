@@ -152,3 +152,28 @@ def test_solver_reports_the_fixed_point_kernel():
         assert pfe.pfe_get_stats(ctx)["filter_shape_f64"] == FIXED
     finally:
         pfe.pfe_destroy(ctx)
+
+
+# ------------------------------------------------------------------ dense products by exact digits
+@pytest.mark.parametrize("width", [48, 63, 64, 65, 127, 128, 129, 200])
+def test_solve_at_widths_around_the_product_tiles(width):
+    """The Gram matrices, projections and block updates of a solve at block widths around the 64 and 128 column
+    tiles: eigenvalues of LAPACK to 1e-10, eigenvectors orthonormal to 1e-12 (a sum of n exact products rounded
+    once, 2^-53, with room for the n = 1,200 of the vectors' own rounding), residuals as the tolerance asks."""
+    g = glassgen.generate(400, 6)
+    ctx = context(g, 0.0)
+    try:
+        H = oracle.csr_from_springs(g)
+        w = np.linalg.eigvalsh(H.dense())
+        lmax, _ = pfe.pfe_estimate(ctx)
+        a, b = 0.5 * (w[9] + w[10]), 0.5 * (w[39] + w[40])
+        pfe.pfe_set_interval(ctx, a, b)
+        pfe.pfe_set_param(ctx, pfe.PFE_P_WIDTH, width)
+        nf, _ = pfe.pfe_solve(ctx)
+        lam, vecs, _ = pfe.pfe_get_eigenpairs(ctx, g.n, nf)
+        assert nf == 30
+        assert np.allclose(lam, w[10:40], rtol=1e-10, atol=0)
+        assert np.max(np.abs(vecs.T @ vecs - np.eye(nf))) <= 1e-12
+        assert np.all(oracle.residuals(H, lam, vecs) <= 1e-8 * lmax)
+    finally:
+        pfe.pfe_destroy(ctx)
