@@ -146,7 +146,14 @@ struct StepArgs {
   int2 ga, gb;           // g_j, g_{j+1} times 2^(kLimb * 2 - 1 - ge), split
   int32_t ge;
   double g0, g1;         // the same coefficients
+  // MODE_EMIT, MODE_ADJ: Y receives the new vector in FP64, times 2^emit
+  int32_t emit;
+  // MODE_ADJ: Z = A X (halved: / 2) - W + g0 Ybar, Ybar in fixed point with its exponents and bounds
+  const int2 *Ybar;
+  const int32_t *ybar_sh, *ybar_mx;
+  int32_t halved;
 };
+constexpr int MODE_EMIT = 5;  // as MODE_STEP, Y = Z
 
 // The FP64 form of the step for one lane's columns (an input with Inf, NaN or extreme magnitudes).
 template <int CPL, int MODE, bool FULL>
@@ -179,9 +186,11 @@ __device__ __noinline__ void raw_step(const StepArgs &a, int64_t atom, int64_t c
     }
     for (int r = 0; r < 3; ++r) {
       const int64_t off = (3 * atom + r) * a.ld + c0 + c;
-      double z = MODE == MODE_FIRST ? 0.5 * acc[r] : acc[r] - W[off];
+      double z = MODE == MODE_FIRST ? 0.5 * acc[r] : (MODE == MODE_ADJ && a.halved ? 0.5 : 1.0) * acc[r] - W[off];
+      if (MODE == MODE_ADJ) z = fma(a.g0, reinterpret_cast<const double *>(a.Ybar)[off], z);
       Z[off] = z;
-      if (MODE == MODE_FIRST) a.Y[off] = fma(a.g1, z, a.g0 * X[off]);
+      if (MODE == MODE_EMIT || MODE == MODE_ADJ) a.Y[off] = ldexp(z, a.emit);
+      else if (MODE == MODE_FIRST) a.Y[off] = fma(a.g1, z, a.g0 * X[off]);
       else if (MODE == MODE_STEP_ACC) a.Y[off] = fma(a.g0, X[off], fma(a.g1, z, a.Y[off]));
       else if (a.Y) a.Y[off] = fma(a.g1, z, a.Y[off]);
     }
@@ -191,10 +200,14 @@ __device__ __noinline__ void raw_step(const StepArgs &a, int64_t atom, int64_t c
 // What the operator allows: the bits of a stored value (64 hold (||A||_inf + 1) of them) and the blocks whose
 // cross terms 64 bits hold.
 __device__ __forceinline__ float norm_of(const int32_t *info) { return fmaxf(__int_as_float(__ldg(info + 1)), 2.f); }
-__device__ __forceinline__ int top_of(float g) { return g < 6.9f ? 60 : g < 14.9f ? 59 : 58; }
-// pairs of rank-1 blocks between two folds
+__device__ __forceinline__ int top_of(const int32_t *info, float g) {
+  const int by_norm = g < 6.9f ? 60 : g < 14.9f ? 59 : 58;
+  // the high limb of u . x takes |u|_1 2^(top - 30) < 2^31
+  return __int_as_float(__ldg(info + 5)) < 1.9f ? by_norm : min(by_norm, 59);
+}
+// rank-1 blocks between two folds
 __device__ __forceinline__ int fold_of(const int32_t *info) {
-  return __int_as_float(__ldg(info + 2)) < 15.5f ? 3 : __int_as_float(__ldg(info + 3)) < 15.5f ? 2 : 1;
+  return __int_as_float(__ldg(info + 2)) < 15.5f ? 6 : __int_as_float(__ldg(info + 3)) < 15.5f ? 4 : 2;
 }
 
 template <int CPL>
@@ -221,15 +234,15 @@ __device__ __forceinline__ void add_block(const int2 (&v)[9], const int2 (&x)[3]
       }
 }
 
-// accH, accM += u (u . x)
+// accH, accM += u (u . x); start: half a unit for the rounding of u . x, plus half a limb so that its low limb comes
+// out signed.  A register: as a constant it costs two additions a column (62 instructions a block instead of 56).
 template <int CPL>
-__device__ __forceinline__ void add_rank1(const int4 &b0, const int4 &b1, const int2 (&x)[3][CPL],
+__device__ __forceinline__ void add_rank1(int64_t start, const int4 &b0, const int4 &b1, const int2 (&x)[3][CPL],
                                           int64_t (&accH)[3][CPL], int64_t (&accM)[3][CPL]) {
   const int2 u[3] = {make_int2(b0.x, b0.y), make_int2(b0.z, b0.w), make_int2(b1.x, b1.y)};
 #pragma unroll
   for (int c = 0; c < CPL; ++c) {
-    // s = u . x rounded, plus half a limb so that its low limb comes out signed
-    int64_t H = mul(u[0].y, x[0][c].y), M = mad(u[0].y, x[0][c].x, (int64_t)kHalf + ((int64_t)kHalf << kLimb));
+    int64_t H = mul(u[0].y, x[0][c].y), M = mad(u[0].y, x[0][c].x, start);
     M = mad(u[0].x, x[0][c].y, M);
 #pragma unroll
     for (int r = 1; r < 3; ++r) {
@@ -249,7 +262,7 @@ __device__ __forceinline__ void add_rank1(const int4 &b0, const int4 &b1, const 
 }
 
 template <int CPL, bool FULL>
-__device__ __forceinline__ void add_neighbour(const int4 *w, const int2 (&x)[3][CPL], int64_t (&accH)[3][CPL],
+__device__ __forceinline__ void add_neighbour(int64_t start, const int4 *w, const int2 (&x)[3][CPL], int64_t (&accH)[3][CPL],
                                               int64_t (&accM)[3][CPL]) {
   if (FULL) {
     int2 v[9];
@@ -261,7 +274,7 @@ __device__ __forceinline__ void add_neighbour(const int4 *w, const int2 (&x)[3][
     v[8] = make_int2(w[4].x, w[4].y);
     add_block<CPL>(v, x, accH, accM);
   } else {
-    add_rank1<CPL>(w[0], w[1], x, accH, accM);
+    add_rank1<CPL>(start, w[0], w[1], x, accH, accM);
   }
 }
 
@@ -287,11 +300,13 @@ struct ColumnScale {
 // memory, so the neighbour loop's only global loads are the gathers, and passes > 1 spreads the set-up over
 // several atoms.
 // What bounds it: IMAD.WIDE runs at about 30 a clock and SM (measured), 18 a block and column make 165 us of the
-// step at N = 99,900, k = 64, and the moves and additions that share its pipe most of the rest; a step moves 614 MB
-// there, 91 us at 6.76 TB/s.  Measured: 876 -> 303 us a step (k = 64), 13.8 -> 4.75 ms (k = 994), full blocks
-// 250 -> 83 us (N = 20,000, k = 64) against the FP64 kernels.  Three CTAs an SM (80 registers): two hide less of
-// the gathers (321 us), four spill (320 us).  Prefetching the next CTAs' rows into L2 gained nothing (340 us), nor
-// did four lanes an atom where the GPU is not full (N = 1,000, k = 16: 8.9 us either way).
+// step at N = 99,900, k = 64, and the moves and additions that share its pipe most of the rest (ncu: that pipe two
+// thirds busy); a step moves 614 MB there, 91 us at 6.76 TB/s.  Measured against the FP64 kernels: 876 -> 280 us a
+// step (k = 64), 13.8 -> 4.37 ms (k = 994), full blocks 250 -> 81 us (N = 20,000, k = 64).
+// 24 warps an SM (80 registers).  Rank-1: CTAs of 128 lanes and one gather at a time; a second gather in flight
+// spills (303 us with 80 registers, 309 with 96), as do 64 registers (296).  Full blocks have three times the
+// products a gather and gain from it (81 against 89 us).  Prefetching rows to L1 or L2 only added instructions
+// (309, 340 us), as did four lanes an atom where the GPU is not full (N = 1,000, k = 16: 8.9 us either way).
 template <int CPL, int MODE, bool FULL>
 __global__ void __launch_bounds__(256, 3) k_fixed_step(const StepArgs a) {
   constexpr int kWords = FULL ? 5 : 2;  // int4 per block
@@ -318,9 +333,13 @@ __global__ void __launch_bounds__(256, 3) k_fixed_step(const StepArgs a) {
     ColumnScale q{};
     float bound = g * (float)(mj + 1);
     bool zero = mj == 0;
-    if (MODE == MODE_FIRST) {
-      bound *= 0.5f;
-    } else {
+    if (MODE == MODE_FIRST || (MODE == MODE_ADJ && a.halved)) bound *= 0.5f;
+    if (MODE == MODE_ADJ) {
+      const int32_t my = a.ybar_mx[c], rel = shj - a.ybar_sh[c];
+      bound += fabsf((float)a.g0) * 1.001f * (float)(my + 1) * __int_as_float((min(max(rel, -126), 90) + 127) << 23);
+      zero = zero && my == 0;
+    }
+    if (MODE != MODE_FIRST) {
       const int32_t mp = a.mx[sp * a.kc + c];
       q.wsh = shj - a.sh[sp * a.kc + c];
       bound += (float)(mp + 1) * __int_as_float((min(max(q.wsh, -126), 90) + 127) << 23);
@@ -328,9 +347,9 @@ __global__ void __launch_bounds__(256, 3) k_fixed_step(const StepArgs a) {
     }
     // bound 1.001 < 2^e: room for top - kLimb - e more bits
     const int e = ((__float_as_int(bound * 1.001f) >> 23) & 255) - 126;
-    const int room = top_of(g) - kLimb - e;
+    const int room = top_of(a.info, g) - kLimb - e;
     q.o = zero ? 0 : room < 0 ? room : room > 1 ? room - 1 : 0;
-    q.ysc = pow2(a.ge + 1 - (shj + q.o));
+    q.ysc = pow2((MODE == MODE_EMIT || MODE == MODE_ADJ ? a.emit : a.ge + 1) - (shj + q.o));
     scale[t] = q;
     if (blockIdx.x == 0) {
       a.sh[sn * a.kc + c] = shj == kRaw ? kRaw : shj + q.o;
@@ -348,10 +367,15 @@ __global__ void __launch_bounds__(256, 3) k_fixed_step(const StepArgs a) {
     plain = plain && sc[c].o == 0 && (MODE == MODE_FIRST || sc[c].wsh == 0);
     big[c] = 0;
   }
+  int64_t start = (int64_t)kHalf + ((int64_t)kHalf << kLimb);
+  asm volatile("" : "+l"(start));
   const int64_t ldb = a.ld * 8;
   const uint32_t stride = (uint32_t)(3 * ldb);
   const char *xl = reinterpret_cast<const char *>(a.X + c0);
   const bool with_y = MODE != MODE_STEP || a.Y != nullptr;
+  int32_t ysh[CPL];
+  if (MODE == MODE_ADJ && !raw)
+    for (int c = 0; c < CPL; ++c) ysh[c] = a.sh[sj * a.kc + c0 + c] - a.ybar_sh[c0 + c] + a.ge + 1;
   for (int32_t atom = first + (int32_t)mine; atom < last; atom += a.per_pass) {
     if (raw) {
       raw_step<CPL, MODE, FULL>(a, atom, c0);
@@ -367,47 +391,60 @@ __global__ void __launch_bounds__(256, 3) k_fixed_step(const StepArgs a) {
       }
     int32_t p = __ldg(a.rp + atom) - pbase;
     const int32_t p1 = __ldg(a.rp + atom + 1) - pbase;
-    // the gather of the next block is in flight during the products of one
-    int2 x0[3][CPL], x1[3][CPL];
+    int2 x0[3][CPL];
     const auto load = [&](int32_t q, int2 (&x)[3][CPL]) {
       load_atom<CPL>(xl, (uint32_t)sblk[q * kWords + kWords - 1].z, stride, ldb, x);
     };
-    if (p < p1) load(p, x0);
-    if (!FULL) {
-      load_atom<CPL>(xl, (uint32_t)atom, stride, ldb, x1);
+    if (FULL) {
+      // the gather of the next block is in flight during the products of one; two blocks between folds
+      int2 x1[3][CPL];
+      if (p < p1) load(p, x0);
+      for (; p + 1 < p1; p += 2) {
+        load(p + 1, x1);
+        add_neighbour<CPL, FULL>(start, sblk + p * kWords, x0, accH, accM);
+        if (p + 2 < p1) load(p + 2, x0);
+        add_neighbour<CPL, FULL>(start, sblk + (p + 1) * kWords, x1, accH, accM);
+        fold<CPL>(accH, accM);
+      }
+      if (p < p1) add_neighbour<CPL, FULL>(start, sblk + p * kWords, x0, accH, accM);
+    } else {
+      load_atom<CPL>(xl, (uint32_t)atom, stride, ldb, x0);
       const int4 d0 = __ldg(a.dg + 3 * (int64_t)atom), d1 = __ldg(a.dg + 3 * (int64_t)atom + 1),
                  d2 = __ldg(a.dg + 3 * (int64_t)atom + 2);
       const int2 xx = make_int2(d0.x, d0.y), xy = make_int2(d0.z, d0.w), xz = make_int2(d1.x, d1.y),
                  yy = make_int2(d1.z, d1.w), yz = make_int2(d2.x, d2.y), zz = make_int2(d2.z, d2.w);
       const int2 v[9] = {xx, xy, xz, xy, yy, yz, xz, yz, zz};
-      add_block<CPL>(v, x1, accH, accM);
-    }
-    const int32_t kFold = FULL ? 1 : fold_of(a.info);
-    int32_t until = kFold;
-    for (; p + 1 < p1; p += 2) {
-      load(p + 1, x1);
-      add_neighbour<CPL, FULL>(sblk + p * kWords, x0, accH, accM);
-      if (p + 2 < p1) load(p + 2, x0);
-      add_neighbour<CPL, FULL>(sblk + (p + 1) * kWords, x1, accH, accM);
-      if (--until == 0) {
-        fold<CPL>(accH, accM);
-        until = kFold;
+      add_block<CPL>(v, x0, accH, accM);
+      const int32_t kFold = fold_of(a.info);
+      int32_t until = kFold;
+      for (; p < p1; ++p) {
+        load(p, x0);
+        add_neighbour<CPL, FULL>(start, sblk + p * kWords, x0, accH, accM);
+        if (--until == 0) {
+          fold<CPL>(accH, accM);
+          until = kFold;
+        }
       }
     }
-    if (p < p1) add_neighbour<CPL, FULL>(sblk + p * kWords, x0, accH, accM);
 #pragma unroll
     for (int r = 0; r < 3; ++r) {
       const int64_t off = (3 * (int64_t)atom + r) * a.ld + c0;
       int2 z[CPL], w[CPL], xo[CPL];
       double y[CPL];
+      constexpr bool kEmit = MODE == MODE_EMIT || MODE == MODE_ADJ;
       if (MODE != MODE_FIRST) load_own<CPL>(a.W + off, w);
       if (MODE == MODE_FIRST || MODE == MODE_STEP_ACC) load_pairs<CPL>(a.X + off, xo);
-      if (MODE != MODE_FIRST && with_y) load_y<CPL>(a.Y + off, y);
+      if (MODE == MODE_ADJ) load_pairs<CPL>(a.Ybar + off, xo);
+      if (MODE != MODE_FIRST && !kEmit && with_y) load_y<CPL>(a.Y + off, y);
 #pragma unroll
       for (int c = 0; c < CPL; ++c) {
         int64_t v = FULL ? (accH[r][c] << 1) + (accM[r][c] >> (kLimb - 1)) : accH[r][c] + (accM[r][c] >> kLimb);
         if (MODE == MODE_FIRST) {
           v = shifted(-v, sc[c].o - 1);
+        } else if (MODE == MODE_ADJ) {
+          const int64_t P = mad(a.ga.y, xo[c].y, mad(a.ga.x, xo[c].y, mad(a.ga.y, xo[c].x, kHalf)) >> kLimb);
+          // each term at the new scale: at the old one g Ybar could exceed 64 bits beside a small a_{j+1}
+          v = shifted(-v, sc[c].o - a.halved) - shifted(join(w[c]), sc[c].wsh + sc[c].o) + shifted(P, ysh[c] + sc[c].o);
         } else if (plain) {
           v = -v - join(w[c]);
         } else {
@@ -415,9 +452,12 @@ __global__ void __launch_bounds__(256, 3) k_fixed_step(const StepArgs a) {
         }
         z[c] = split(v);
         big[c] = max(big[c], abs(z[c].y));
+        if (kEmit) y[c] = to_double(v) * sc[c].ysc;
       }
       store_pairs<CPL>(a.Z + off, z);
-      if (with_y) {
+      if (kEmit) {
+        store_y<CPL>(a.Y + off, y);
+      } else if (with_y) {
 #pragma unroll
         for (int c = 0; c < CPL; ++c) {
           int64_t H = mad(a.gb.y, z[c].y, 0), M = mad(a.gb.x, z[c].y, mad(a.gb.y, z[c].x, kHalf));
@@ -442,7 +482,11 @@ __global__ void __launch_bounds__(256, 3) k_fixed_step(const StepArgs a) {
 }
 
 // ---- the operator in fixed point -------------------------------------------------------------
-__device__ __forceinline__ int2 fixed_entry(double v, double unit) { return split(__double2ll_rn(v * unit)); }
+__device__ __forceinline__ int2 fixed_entry(double v, double unit) {
+  const int64_t t = __double2ll_rn(v * unit);
+  // +2 in units of 2^-60 (an atom without neighbours): one limb down from 2^31
+  return t > ((int64_t)1 << 61) - kHalf - 1 ? make_int2((int32_t)(t - ((int64_t)INT32_MAX << kLimb)), INT32_MAX) : split(t);
+}
 
 // info[0] |= 1 when the operator does not fit; info[1]: ||A||_inf as float bits, rounded up
 __device__ __forceinline__ void note_row(int32_t *info, double row, bool bad) {
@@ -452,7 +496,8 @@ __device__ __forceinline__ void note_row(int32_t *info, double row, bool bad) {
 
 // Rank-1 form, unit 2^-60.  With |x| < 2^60 the cross terms of a row's diagonal block and F of its other blocks
 // stay below 2^59 (3 + sum |d| + sum (|u_r| + |u|_1)): info[2], info[3] get the largest such factor for F = 6, 4
-// (below 15.5: 63 bits hold them; F = 2 always does).
+// (below 15.5: 63 bits hold them; F = 2 always does).  info[4]: the
+// longest row, info[5]: the largest |u|_1.
 __global__ void k_fixed_r1(int32_t n_atoms, const int32_t *__restrict__ rp1, const int32_t *__restrict__ ci1,
                            const double *__restrict__ u, const double *__restrict__ dg, int4 *blk, int2 *dgo,
                            int32_t *info) {
@@ -463,19 +508,20 @@ __global__ void k_fixed_r1(int32_t n_atoms, const int32_t *__restrict__ rp1, con
                    fabs(d[2]) + fabs(d[4]) + fabs(d[5])};
   bool bad = !(row[0] < 4.0 && row[1] < 4.0 && row[2] < 4.0);
   for (int t = 0; t < 6; ++t) {
-    bad = bad || !(fabs(d[t]) < 1.99);
+    bad = bad || !(fabs(d[t]) <= 2.0);
     dgo[6 * i + t] = bad ? make_int2(0, 0) : fixed_entry(-d[t], 0x1p60);
   }
   const double drow = fmax(row[0], fmax(row[1], row[2]));
-  double s6[3] = {0, 0, 0}, s4[3] = {0, 0, 0}, m6 = 0.0, m4 = 0.0;
+  double s6[3] = {0, 0, 0}, s4[3] = {0, 0, 0}, m6 = 0.0, m4 = 0.0, u1 = 0.0;
   const int32_t p0 = rp1[i], p1 = rp1[i + 1];
   for (int32_t p = p0; p < p1 && !bad; ++p) {
     const double v[3] = {u[3 * (int64_t)p], u[3 * (int64_t)p + 1], u[3 * (int64_t)p + 2]};
     const double s = fabs(v[0]) + fabs(v[1]) + fabs(v[2]);
-    if (!(s < 1.9)) {  // u . x has to stay below 2^61 for |x| < 2^60
+    if (!(fmax(fabs(v[0]), fmax(fabs(v[1]), fabs(v[2]))) < 1.99)) {  // a limb is 31 bits; |u|_2 <= sqrt(2) when ||A|| <= 2
       bad = true;
       break;
     }
+    u1 = fmax(u1, s);
     const bool new6 = (p - p0) % 6 == 0, new4 = (p - p0) % 4 == 0;
     for (int r = 0; r < 3; ++r) {
       row[r] += fabs(v[r]) * s;
@@ -491,6 +537,7 @@ __global__ void k_fixed_r1(int32_t n_atoms, const int32_t *__restrict__ rp1, con
   if (!bad) {
     atomicMax(info + 2, __float_as_int((float)(3.0 + drow + m6)));
     atomicMax(info + 3, __float_as_int((float)(3.0 + drow + m4)));
+    atomicMax(info + 5, __float_as_int((float)u1));
   }
   atomicMax(info + 4, p1 - p0);
   note_row(info, fmax(row[0], fmax(row[1], row[2])), bad);
@@ -578,7 +625,7 @@ __global__ void k_fixed_plan(int32_t k, int32_t parts, const uint64_t *__restric
       continue;
     }
     const float g = norm_of(info);
-    s0[t] = top_of(g) - 1 - ilogb(v * ((double)g + 1.0) * 1.0001);
+    s0[t] = top_of(info, g) - 1 - ilogb(v * ((double)g + 1.0) * 1.0001);
     m0[t] = (int32_t)ldexp(v, s0[t] - kLimb) + 1;
   }
   for (int t = 0; t < cpl; ++t) {
@@ -635,6 +682,10 @@ void launch_step(int mode, const StepArgs &a, dim3 grid, int threads, size_t sme
     PFE_LAUNCH k_fixed_step<CPL, MODE_FIRST, FULL><<<grid, threads, smem, s>>>(a);
   else if (mode == MODE_STEP_ACC)
     PFE_LAUNCH k_fixed_step<CPL, MODE_STEP_ACC, FULL><<<grid, threads, smem, s>>>(a);
+  else if (mode == MODE_EMIT)
+    PFE_LAUNCH k_fixed_step<CPL, MODE_EMIT, FULL><<<grid, threads, smem, s>>>(a);
+  else if (mode == MODE_ADJ)
+    PFE_LAUNCH k_fixed_step<CPL, MODE_ADJ, FULL><<<grid, threads, smem, s>>>(a);
   else
     PFE_LAUNCH k_fixed_step<CPL, MODE_STEP, FULL><<<grid, threads, smem, s>>>(a);
 }
@@ -669,38 +720,25 @@ bool fixed_coefficients_ok(const double *coef, int32_t m) {
   return m >= 1 && g < 0x1p60;
 }
 
-void launch_fixed_filter(const Bsr<double> &A, const FixedOp &op, const double *coef, int32_t m, int32_t k, int64_t ld,
-                         const double *X, int64_t ldx, bool colmajor, double *Y, double *b0, double *b1, void *state,
-                         cudaStream_t s) {
-  const int64_t n = 3 * (int64_t)A.n_atoms, kc = (k + 3) / 4 * 4;
-  int32_t *sh = static_cast<int32_t *>(state), *mx = sh + 4 * kc;
-  uint64_t *part = reinterpret_cast<uint64_t *>(mx + 4 * kc);
-  auto al16 = [](const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
+namespace {
+
+// What the steps of one call share: the operator, the lanes and the CTA shape
+struct StepPlan {
+  StepArgs a{};
+  bool rank1 = false;
+  int cpl = 1, threads = 0;
+  size_t smem = 0;
+  dim3 grid;
+};
+
+StepPlan plan_steps(const Bsr<double> &A, const FixedOp &op, int32_t k, int64_t ld, bool aligned) {
+  StepPlan p;
+  p.rank1 = A.u != nullptr;
   // Two columns a lane (16-byte gathers) once the lanes fill the GPU a few times over; before that one, for more
   // lanes (N = 1,000, k = 16: 9.0 us a step with one, 12.0 with two; N = 5,003, k = 33: 19.8 and 20.7;
   // N = 99,900, k = 64: 334 and 303).
-  const bool wide = k > 1 && ld % 2 == 0 && al16(Y) && al16(b0) && al16(b1);
-  const int cpl = wide && (int64_t)A.n_atoms * k >= 200000 ? 2 : 1;
-  const int32_t npc = (k + cpl - 1) / cpl, kp = npc * cpl;
-  // exponents of t_0 and its conversion into b1
-  const int32_t parts = max_parts(n);
-  const int64_t slab = (n + parts - 1) / parts;
-  const uint64_t *xb = reinterpret_cast<const uint64_t *>(X);
-  int2 *t0 = reinterpret_cast<int2 *>(b1), *t1 = reinterpret_cast<int2 *>(b0);
-  if (colmajor)
-    PFE_LAUNCH k_colmax_cm<<<dim3(parts, std::min(k, 65535)), 256, 0, s>>>(n, k, xb, ldx, slab, part);
-  else
-    PFE_LAUNCH k_colmax_rm<<<dim3(parts, (k + 31) / 32), 256, 0, s>>>(n, k, xb, ldx, slab, part);
-  PFE_LAUNCH k_fixed_plan<<<(unsigned)((kc / cpl + 127) / 128), 128, 0, s>>>(k, parts, part, cpl, op.info, kc, sh, mx);
-  if (colmajor)
-    PFE_LAUNCH k_fixed_from_cm<<<dim3((unsigned)((n + 31) / 32), (kp + 31) / 32), 256, 0, s>>>(n, k, kp, xb, ldx, sh, t0, ld);
-  else
-    PFE_LAUNCH k_fixed_from_rm<<<(unsigned)((n * kp + 255) / 256), 256, 0, s>>>(n, k, kp, xb, ldx, sh, t0);
-  auto fixed = [](double v, int ge) {  // v 2^(59 - ge), split; |v| <= 2^ge
-    const int64_t t = std::llrint(std::ldexp(v, 2 * kLimb - 1 - ge)) + kHalf;
-    return make_int2((int32_t)(t & kMask) - kHalf, (int32_t)(t >> kLimb));
-  };
-  StepArgs a{};
+  p.cpl = aligned && k > 1 && ld % 2 == 0 && (int64_t)A.n_atoms * k >= 200000 ? 2 : 1;
+  StepArgs &a = p.a;
   a.n_atoms = A.n_atoms;
   a.ld = ld;
   a.rp = A.u ? A.rp1 : A.rp;
@@ -710,47 +748,186 @@ void launch_fixed_filter(const Bsr<double> &A, const FixedOp &op, const double *
   a.d64 = A.dg;
   a.ci64 = A.u ? A.ci1 : A.ci;
   a.info = op.info;
-  a.sh = sh;
-  a.mx = mx;
-  a.kc = kc;
-  // CTA shape: the fewest column tiles, evenly wide; as many atoms at a time as 256 lanes hold; up to four passes
-  // while every SM keeps its three CTAs (N = 99,900, k = 64: 318 us a step with one pass, 303 with four, 302 with
-  // eight; N = 5,003, k = 33: 20.7 with one, 24.9 with four).
-  const int tiles = (npc + 255) / 256;
+  a.kc = (k + 3) / 4 * 4;
+  // CTA shape: the fewest column tiles, evenly wide.  Rank-1: as many atoms at a time as 128 lanes hold, more where
+  // whole warps then waste fewer lanes (k = 33: 99 of 128 or 231 of 256; N = 5,003: 21.9 and 20.0 us a step); full
+  // blocks: 256 lanes.  Up to four passes while every SM keeps its CTAs (N = 99,900, k = 64: 318 us a step with one pass, 303 with four, 302 with eight;
+  // N = 5,003, k = 33: 20.7 with one, 24.9 with four).
+  const int32_t npc = (k + p.cpl - 1) / p.cpl;
+  const int lanes = A.u ? 128 : 256;
+  const int tiles = (npc + lanes - 1) / lanes;
   a.groups = npc;
   a.tile = (npc + tiles - 1) / tiles;
-  a.per_pass = 256 / a.tile;
+  const auto used = [&](int atoms) {  // share of the lanes, less a little for the larger CTAs
+    const int t = (atoms * a.tile + 31) / 32 * 32;
+    return (double)(atoms * a.tile) / t * (t <= lanes ? 1.0 : 0.95);
+  };
+  a.per_pass = lanes / a.tile;
+  for (int atoms = a.per_pass + 1; atoms * a.tile <= 256; ++atoms)
+    if (used(atoms) > used(a.per_pass)) a.per_pass = atoms;
   a.magic = (65536 + a.tile - 1) / a.tile;
   const size_t row_bytes = (size_t)op.max_row * fixed_block_bytes(A);
   while (a.per_pass > 1 && a.per_pass * row_bytes > kFixedStage) --a.per_pass;
-  const int threads = (a.per_pass * a.tile + 31) / 32 * 32;
+  p.threads = (a.per_pass * a.tile + 31) / 32 * 32;
   const int64_t ctas = ((int64_t)A.n_atoms + a.per_pass - 1) / a.per_pass * tiles;
-  a.passes = (int32_t)std::min<int64_t>(4, std::max<int64_t>(1, ctas / (3 * 152)));
+  a.passes = (int32_t)std::min<int64_t>(4, std::max<int64_t>(1, ctas * p.threads / (768 * 152)));
   while (a.passes > 1 && a.per_pass * a.passes * row_bytes > kFixedStage) --a.passes;
   const int per_cta = a.per_pass * a.passes;
-  const size_t smem = (size_t)a.tile * cpl * sizeof(ColumnScale) + per_cta * row_bytes;
-  const dim3 grid((unsigned)((A.n_atoms + per_cta - 1) / per_cta), (unsigned)tiles);
+  p.smem = (size_t)a.tile * p.cpl * sizeof(ColumnScale) + per_cta * row_bytes;
+  p.grid = dim3((unsigned)((A.n_atoms + per_cta - 1) / per_cta), (unsigned)tiles);
+  return p;
+}
+
+void launch_planned(const StepPlan &p, int mode, cudaStream_t s) {
+  if (p.rank1) {
+    if (p.cpl == 2) launch_step<2, false>(mode, p.a, p.grid, p.threads, p.smem, s);
+    else launch_step<1, false>(mode, p.a, p.grid, p.threads, p.smem, s);
+  } else {
+    if (p.cpl == 2) launch_step<2, true>(mode, p.a, p.grid, p.threads, p.smem, s);
+    else launch_step<1, true>(mode, p.a, p.grid, p.threads, p.smem, s);
+  }
+}
+
+// v 2^(59 - ge), split; |v| <= 2^ge
+int2 fixed_coefficient(double v, int ge) {
+  const int64_t t = std::llrint(std::ldexp(v, 2 * kLimb - 1 - ge)) + kHalf;
+  return make_int2((int32_t)(t & kMask) - kHalf, (int32_t)(t >> kLimb));
+}
+int coefficient_exponent(double g) { return g != 0.0 ? std::ilogb(g) + 1 : 0; }
+
+// exponents and bounds of a block's columns (slots 0 and 1 of sh and mx)
+void plan_columns(const StepPlan &p, int64_t n, int32_t k, const double *X, int64_t ldx, bool colmajor, int32_t *sh,
+                  int32_t *mx, uint64_t *part, cudaStream_t s) {
+  const int32_t parts = max_parts(n);
+  const int64_t slab = (n + parts - 1) / parts;
+  const uint64_t *xb = reinterpret_cast<const uint64_t *>(X);
+  if (colmajor)
+    PFE_LAUNCH k_colmax_cm<<<dim3(parts, std::min(k, 65535)), 256, 0, s>>>(n, k, xb, ldx, slab, part);
+  else
+    PFE_LAUNCH k_colmax_rm<<<dim3(parts, (k + 31) / 32), 256, 0, s>>>(n, k, xb, ldx, slab, part);
+  PFE_LAUNCH k_fixed_plan<<<(unsigned)((p.a.kc / p.cpl + 127) / 128), 128, 0, s>>>(k, parts, part, p.cpl, p.a.info, p.a.kc,
+                                                                                  sh, mx);
+}
+
+void convert_columns(const StepPlan &p, int64_t n, int32_t k, const double *X, int64_t ldx, bool colmajor,
+                     const int32_t *sh, int2 *T, cudaStream_t s) {
+  const int32_t kp = p.a.groups * p.cpl;
+  const uint64_t *xb = reinterpret_cast<const uint64_t *>(X);
+  if (colmajor)
+    PFE_LAUNCH k_fixed_from_cm<<<dim3((unsigned)((n + 31) / 32), (kp + 31) / 32), 256, 0, s>>>(n, k, kp, xb, ldx, sh, T,
+                                                                                             p.a.ld);
+  else
+    PFE_LAUNCH k_fixed_from_rm<<<(unsigned)((n * kp + 255) / 256), 256, 0, s>>>(n, k, kp, xb, ldx, sh, T);
+}
+
+bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
+
+// a_m and Ybar of the adjoint: a column kept in FP64 on one side is so on both; a zero a_m takes Ybar's exponent;
+// slot 3 is a_{m+1} = 0
+__global__ void k_fixed_adjoint_columns(int64_t kc, int cpl, int32_t *sh, int32_t *mx, int32_t *ysh, const int32_t *ymx) {
+  const int64_t c0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * cpl;
+  if (c0 >= kc) return;
+  bool raw = false;
+  for (int t = 0; t < cpl; ++t) raw = raw || sh[c0 + t] == kRaw || ysh[c0 + t] == kRaw;
+  for (int t = 0; t < cpl; ++t) {
+    const int64_t c = c0 + t;
+    if (raw) sh[c] = ysh[c] = kRaw;
+    else if (mx[c] == 0 && ymx[c] != 0) sh[c] = ysh[c];
+    sh[3 * kc + c] = sh[c];
+    mx[3 * kc + c] = 0;
+  }
+}
+
+}  // namespace
+
+void launch_fixed_filter(const Bsr<double> &A, const FixedOp &op, const double *coef, int32_t m, int32_t k, int64_t ld,
+                         const double *X, int64_t ldx, bool colmajor, double *Y, double *b0, double *b1, void *state,
+                         cudaStream_t s) {
+  const int64_t n = 3 * (int64_t)A.n_atoms;
+  StepPlan p = plan_steps(A, op, k, ld, aligned16(Y) && aligned16(b0) && aligned16(b1));
+  StepArgs &a = p.a;
+  a.sh = static_cast<int32_t *>(state);
+  a.mx = a.sh + 4 * a.kc;
+  int2 *t0 = reinterpret_cast<int2 *>(b1), *t1 = reinterpret_cast<int2 *>(b0);
+  plan_columns(p, n, k, X, ldx, colmajor, a.sh, a.mx, reinterpret_cast<uint64_t *>(a.mx + 4 * a.kc), s);
+  convert_columns(p, n, k, X, ldx, colmajor, a.sh, t0, s);
   for (int32_t j = 0; j < m; ++j) {
     // y takes two terms every other step, as in the FP64 filter
     const bool even = (j % 2) == 0, last = j == m - 1;
-    const int mode = j == 0 ? MODE_FIRST : even ? MODE_STEP_ACC : MODE_STEP;
     a.j = j;
     a.X = even ? t0 : t1;
     a.W = a.Z = even ? t1 : t0;
     a.Y = (even || last) ? Y : nullptr;
-    const double g = std::fmax(even ? std::fabs(coef[j]) : 0.0, std::fabs(coef[j + 1]));
-    a.ge = g > 0.0 ? std::ilogb(g) + 1 : 0;  // the pair's own exponent: a small pair keeps its relative accuracy
-    a.ga = even ? fixed(coef[j], a.ge) : make_int2(0, 0);
-    a.gb = fixed(coef[j + 1], a.ge);
+    // the pair's own exponent: a small pair keeps its relative accuracy
+    a.ge = coefficient_exponent(std::fmax(even ? std::fabs(coef[j]) : 0.0, std::fabs(coef[j + 1])));
+    a.ga = even ? fixed_coefficient(coef[j], a.ge) : make_int2(0, 0);
+    a.gb = fixed_coefficient(coef[j + 1], a.ge);
     a.g0 = coef[j];
     a.g1 = coef[j + 1];
-    if (A.u) {
-      if (cpl == 2) launch_step<2, false>(mode, a, grid, threads, smem, s);
-      else launch_step<1, false>(mode, a, grid, threads, smem, s);
-    } else {
-      if (cpl == 2) launch_step<2, true>(mode, a, grid, threads, smem, s);
-      else launch_step<1, true>(mode, a, grid, threads, smem, s);
+    launch_planned(p, j == 0 ? MODE_FIRST : even ? MODE_STEP_ACC : MODE_STEP, s);
+  }
+}
+
+size_t fixed_adjoint_state_bytes(int64_t n, int32_t k) {
+  return fixed_state_bytes(n, k) + (size_t)(4 * ((k + 3) / 4 * 4)) * sizeof(int32_t);
+}
+
+void launch_fixed_adjoint(const Bsr<double> &A, const FixedOp &op, const double *coef, int32_t m, int32_t k, int64_t ld,
+                          const double *Ybar, double *t, double *adj, double *b0, double *b1, double *b2, void *state,
+                          cudaStream_t s) {
+  const int64_t n = 3 * (int64_t)A.n_atoms, vec = n * ld;
+  StepPlan p = plan_steps(A, op, k, ld, aligned16(t) && aligned16(adj) && aligned16(b0) && aligned16(b1) && aligned16(b2) && vec % 2 == 0);
+  StepArgs &a = p.a;
+  a.sh = static_cast<int32_t *>(state);
+  a.mx = a.sh + 4 * a.kc;
+  int32_t *ysh = a.mx + 4 * a.kc, *ymx = ysh + 2 * a.kc;
+  uint64_t *part = reinterpret_cast<uint64_t *>(ymx + 2 * a.kc);
+  int2 *v0 = reinterpret_cast<int2 *>(b0), *v1 = reinterpret_cast<int2 *>(b1), *yb = reinterpret_cast<int2 *>(b2);
+  // t_1 .. t_{m-1}
+  if (m > 1) {
+    plan_columns(p, n, k, t, ld, false, a.sh, a.mx, part, s);
+    convert_columns(p, n, k, t, ld, false, a.sh, v0, s);
+    for (int32_t j = 0; j + 1 < m; ++j) {
+      a.j = j;
+      a.X = j % 2 == 0 ? v0 : v1;
+      a.W = a.Z = j % 2 == 0 ? v1 : v0;
+      a.Y = t + (j + 1) * vec;
+      a.emit = 0;
+      a.ge = 1;  // MODE_FIRST: y = 0 x + 1 t_1
+      a.ga = make_int2(0, 0);
+      a.gb = fixed_coefficient(1.0, 1);
+      a.g0 = 0.0;
+      a.g1 = 1.0;
+      launch_planned(p, j == 0 ? MODE_FIRST : MODE_EMIT, s);
     }
+  }
+  // a_{m-1} .. a_0 from a_m = g_m Ybar; the coefficients scaled to at most 1 so that tiny ones keep their accuracy
+  double top = 0.0;
+  for (int32_t j = 0; j <= m; ++j) top = std::fmax(top, std::fabs(coef[j]));
+  const int up = coefficient_exponent(top);
+  launch_axpby<double>(n, k, std::ldexp(coef[m], -up), Ybar, ld, 0.0, adj + m * vec, ld, s);
+  plan_columns(p, n, k, Ybar, ld, false, ysh, ymx, part, s);
+  plan_columns(p, n, k, adj + m * vec, ld, false, a.sh, a.mx, part, s);
+  PFE_LAUNCH k_fixed_adjoint_columns<<<(unsigned)((a.kc / p.cpl + 127) / 128), 128, 0, s>>>(a.kc, p.cpl, a.sh, a.mx, ysh, ymx);
+  convert_columns(p, n, k, Ybar, ld, false, ysh, yb, s);
+  convert_columns(p, n, k, adj + m * vec, ld, false, a.sh, v0, s);
+  cudaMemsetAsync(v1, 0, (size_t)vec * sizeof(int2), s);
+  launch_axpby<double>(n, k, coef[m], Ybar, ld, 0.0, adj + m * vec, ld, s);
+  a.Ybar = yb;
+  a.ybar_sh = ysh;
+  a.ybar_mx = ymx;
+  a.emit = up;
+  for (int32_t r = 0; r < m; ++r) {
+    const int32_t j = m - 1 - r;
+    a.j = r;
+    a.X = r % 2 == 0 ? v0 : v1;
+    a.W = a.Z = r % 2 == 0 ? v1 : v0;
+    a.Y = adj + j * vec;
+    a.halved = j == 0;
+    a.g0 = std::ldexp(coef[j], -up);
+    a.ge = coefficient_exponent(a.g0);
+    a.ga = fixed_coefficient(a.g0, a.ge);
+    launch_planned(p, MODE_ADJ, s);
   }
 }
 

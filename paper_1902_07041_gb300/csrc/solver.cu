@@ -1814,6 +1814,27 @@ pfe_status pfe_filter_adjoint(pfe_ctx *ctx, int32_t m, const double *coeffs, int
   if (k == 0) return check_launch(ctx, "filter_adjoint");
   const int64_t n = ctx->n, ld = round_up(k, 2);
   const size_t vec = (size_t)n * ld;
+  const Bsr<double> A = bsr_Hs64(ctx);
+  const double two_over_d = 2.0 / ctx->td;
+  // In fixed point with every t_j and a_j kept (no recomputation) while they take at most 16 GB; a device without
+  // that room, an operator that does not fit and larger problems take the checkpoints below.
+  if (m >= 1 && step_variant(0) < 0 && fixed_coefficients_ok(cf, m) && (2 * (size_t)m + 6) * vec * sizeof(double) <= ((size_t)16 << 30)) {
+    PFE_TRY(ensure_fixed(ctx, A));
+    const FixedOp op = solver_fixed_op(ctx, cf, m);
+    const size_t state_bytes = (fixed_adjoint_state_bytes(n, k) + 255) / 256 * 256;
+    if (op.blocks && dbuf_reserve(ctx->w_ckpt, state_bytes + (2 * (size_t)m + 6) * vec * sizeof(double)) == cudaSuccess) {
+      void *state = ctx->w_ckpt.p;
+      double *t = reinterpret_cast<double *>(static_cast<char *>(state) + state_bytes), *adj = t + (size_t)m * vec;
+      double *Yb = adj + ((size_t)m + 1) * vec, *b0 = Yb + vec, *b1 = b0 + vec, *b2 = b1 + vec;
+      launch_colmajor_to_rowmajor<double>(n, k, X, ldx, t, ld, s);
+      launch_colmajor_to_rowmajor<double>(n, k, Ybar, ldyb, Yb, ld, s);
+      launch_fixed_adjoint(A, op, cf, m, k, ld, Yb, t, adj, b0, b1, b2, state, s);
+      launch_outer_accum_seg(A, ctx->nnzb, k, ld, m, (int64_t)vec, adj + vec, t, 0.5 * two_over_d, two_over_d, vals_bar, s);
+      launch_rowmajor_to_colmajor<double>(n, k, adj, ld, Xbar, ldxb, s);
+      return check_launch(ctx, "filter_adjoint");
+    }
+    cudaGetLastError();  // a failed allocation's error state
+  }
   // checkpoint spacing ~ sqrt(m): checkpoints hold (t_j0, t_{j0+1}) for j0 = 0, S, 2S, ...
   const int32_t S = std::max<int32_t>(1, (int32_t)std::ceil(std::sqrt((double)std::max(m, 1))));
   const int32_t nseg = (m + S - 1) / S;
@@ -1827,8 +1848,6 @@ pfe_status pfe_filter_adjoint(pfe_ctx *ctx, int32_t m, const double *coeffs, int
   launch_zero<double>(base, (int64_t)(vec * nvec), s);
   launch_colmajor_to_rowmajor<double>(n, k, X, ldx, Xr, ld, s);
   launch_colmajor_to_rowmajor<double>(n, k, Ybar, ldyb, Yb, ld, s);
-  const Bsr<double> A = bsr_Hs64(ctx);
-  const double two_over_d = 2.0 / ctx->td;
   auto tvec = [&](int32_t g, int which) { return ck + ((size_t)2 * g + which) * vec; };
   auto av = [&](int32_t q) { return aseg + (size_t)q * vec; };
   // forward pass: t_0 .. t_{m-1}, storing (t_j0, t_{j0+1}) at every segment start j0 = g S

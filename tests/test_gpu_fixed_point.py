@@ -129,6 +129,36 @@ def test_fixed_point_filter_rescales_growing_vectors(rank1):
         pfe.pfe_destroy(ctx)
 
 
+def test_atoms_without_neighbours_and_stiff_bonds():
+    """A bond far stiffer than the others along (1, 1, 1) (|u|_1 near its bound) and an atom without bonds (a diagonal
+    entry of exactly -2): both still fit."""
+    g = glassgen.generate(300, 4)
+    keep = (g.bi != 17) & (g.bj != 17)
+    bi, bj, k, rhat = g.bi[keep], g.bj[keep], g.k[keep].copy(), g.rhat[keep].copy()
+    k[40], rhat[40] = 60.0, np.ones(3) / np.sqrt(3.0)
+    rp, ci, vals = pfe.pfe_springs_to_bsr(g.n_atoms, bi, bj, k, rhat)
+    H = np.zeros((g.n, g.n))
+    for i in range(g.n_atoms):
+        for p in range(rp[i], rp[i + 1]):
+            H[3 * i:3 * i + 3, 3 * ci[p]:3 * ci[p] + 3] = vals[9 * p:9 * p + 9].reshape(3, 3) / np.sqrt(g.mass[i] * g.mass[ci[p]])
+    lmax = 1.0001 * np.linalg.eigvalsh(H)[-1]
+    ctx = pfe.pfe_create(g.n_atoms, rp, ci, vals, g.mass)
+    pfe.pfe_set_param(ctx, pfe.PFE_P_LAMBDA_MAX, lmax)
+    try:
+        coef = np.array([0.1, 0.2, -0.3, 0.4, 0.5, -0.1])
+        X = np.random.default_rng(5).standard_normal((g.n, 7))
+        Y = apply(ctx, coef, X)
+        T = [X, 2.0 / lmax * (H @ X) - X]
+        for _ in coef[2:]:
+            T.append(2.0 * (2.0 / lmax * (H @ T[-1]) - T[-1]) - T[-2])
+        ref = sum(c * t for c, t in zip(coef, T))
+        assert np.max(np.abs(Y - ref)) <= tolerance(X, coef)
+        Y2 = apply(ctx, coef, X, shape=7)
+        assert np.any(Y != Y2)  # the two kernels round differently: the fixed-point one ran
+    finally:
+        pfe.pfe_destroy(ctx)
+
+
 def test_operator_that_does_not_fit_runs_in_fp64():
     """An operator with entries beyond the fixed-point range (a bound far below the spectrum) keeps the FP64 kernels."""
     g = glassgen.generate(200, 4)
@@ -176,4 +206,46 @@ def test_solve_at_widths_around_the_product_tiles(width):
         assert np.max(np.abs(vecs.T @ vecs - np.eye(nf))) <= 1e-12
         assert np.all(oracle.residuals(H, lam, vecs) <= 1e-8 * lmax)
     finally:
+        pfe.pfe_destroy(ctx)
+
+
+# ------------------------------------------------------------------ the adjoint
+@pytest.mark.parametrize("rank1", [1, 0])
+@pytest.mark.parametrize("N,k,coef", [(60, 1, [0.5, 0.25]), (61, 2, [0.5, 0.25, 1e-17]), (333, 5, [0.0, 0.3, -0.2, 0.1, 0.0]),
+                                      (300, 129, [1e-9, 2e-9, -3e-9, 1e-9]), (4001, 52, [0.1, -0.4, 0.3, 0.2, 0.05, 1e-3])])
+def test_fixed_point_adjoint_matches_the_checkpointed_one(N, k, coef, rank1):
+    """The adjoint that keeps every vector, in fixed point, against the FP64 kernels with checkpoints (a forced kernel
+    shape): one step to several, odd and single columns, a last coefficient of 0 or far below the others, columns of
+    0, Inf and very small entries beside ordinary ones.  Tolerance as for the filter, with the products' sums of k m
+    terms beside it."""
+    g = glassgen.generate(N, 9)
+    ctx = context(g, 0.25, rank1)
+    try:
+        coef = np.array(coef)
+        m = coef.size - 1
+        rng = np.random.default_rng(N)
+        X, Yb = rng.standard_normal((g.n, k)), rng.standard_normal((g.n, k))
+        if k > 4:
+            X[:, 1] = 0.0
+            Yb[:, 2] = 0.0
+            Yb[:, 3] *= 1e-295
+        rp, ci, _ = pfe.pfe_springs_to_bsr(g.n_atoms, g.bi, g.bj, g.k, g.rhat)
+        got = []
+        for shape in (-1, 7 if rank1 else 0):
+            Xd, Yd = (torch.from_numpy(np.ascontiguousarray(v.T)).cuda() for v in (X, Yb))
+            Xb, vb = torch.empty_like(Xd), torch.empty(9 * ci.size, dtype=torch.float64, device="cuda")
+            pfe.pfe_set_param(ctx, pfe.PFE_P_STEP_SHAPE_F64, shape)
+            pfe.pfe_filter_adjoint(ctx, m, coef, k, Xd, g.n, Yd, g.n, Xb, g.n, vb)
+            torch.cuda.synchronize()
+            pfe.pfe_set_param(ctx, pfe.PFE_P_STEP_SHAPE_F64, -1)
+            got.append((Xb.cpu().numpy().T, vb.cpu().numpy()))
+        tol = tolerance(Yb, coef)
+        assert np.max(np.abs(got[0][0] - got[1][0])) <= tol
+        assert np.max(np.abs(got[0][1] - got[1][1])) <= 2.0 / 0.125 * k * tol * np.linalg.norm(X, axis=0).max()
+        if k > 4:
+            assert not got[0][0][:, 2].any()
+            small = got[1][0][:, 3]
+            assert np.max(np.abs(got[0][0][:, 3] - small)) <= 1e-12 * np.abs(small).max()
+    finally:
+        pfe.pfe_set_param(ctx, pfe.PFE_P_STEP_SHAPE_F64, -1)
         pfe.pfe_destroy(ctx)
