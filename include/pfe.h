@@ -249,7 +249,7 @@ typedef struct {
   int64_t filter_col_steps;    /* sum over those launches of their column counts (FP64 filter) */
   int64_t filter_col_steps_f32;/* the same for the FP32 filter */
   double seconds_filter_f32;   /* part of seconds_filter spent in FP32 filter sweeps */
-  int64_t batch_replays;       /* pfe_solve_batch: replays of the captured batched-filter graph */
+  int64_t batch_replays;       /* pfe_solve_batch: filter applications (the most that a sample took) */
   int32_t restarts;            /* METHOD 1: thick restarts */
   int32_t basis;               /* METHOD 1: maximal basis size */
   int32_t filter_shape_f64;    /* kernel shape of the last FP64 filter step (PFE_P_STEP_SHAPE_F64 numbering;
@@ -343,18 +343,21 @@ pfe_status pfe_probe_fp64_fma(int32_t iters, int32_t reps, void *stream, double 
  * ------------------------------------------------------------------------------------- */
 
 /* Solve every context's interval problem; n_found[s] per sample.  Each context must have its
- * interval set; all must live on one device.  The iterations of all samples advance in lockstep:
- * the filter of every FP64 sample runs as one persistent kernel per Chebyshev step over all
- * samples' work, captured once in a CUDA graph and replayed per iteration (its column tile and
- * grid size chosen by timing the candidates on the first call); the dense steps run per sample,
- * the samples' dense steps concurrently from PFE_P_BATCH_THREADS host threads.  When every context
+ * interval set; all must live on one device.  Samples whose filter runs in fixed point or in FP32
+ * iterate independently, each on its own stream, from PFE_P_BATCH_THREADS host threads.  While some
+ * sample's FP64 filter cannot run in fixed point (a forced kernel shape, degree 0, an operator that
+ * does not fit), all samples advance in lockstep: the filters of those run as one persistent kernel
+ * per Chebyshev step over their work, captured once in a CUDA graph and replayed per iteration (its
+ * column tile and grid size chosen by timing the candidates on the first call), the rest per sample,
+ * concurrently from the same threads.  When every context
  * selects PFE_P_METHOD = 1 the samples' block Lanczos solves run whole, concurrently from those
  * threads, each on its own stream, largest samples first; a finished sample's work buffers pass to
  * the next sample its thread solves (its eigenvectors stay), so only the solves in flight hold them
  * and none is freed while others run, and a sample that ran out of device memory beside the others
  * is solved again afterwards, alone.  All contexts of a batch select the same method (PFE_E_ARG otherwise).
- * In the stats of every sample seconds_filter is the batch's shared filter time.  In the lockstep
- * subspace iteration too, a sample that ran out of device memory beside the others is solved again
+ * In the stats of every sample seconds_filter is the batch's filter time: the shared launches' in
+ * lockstep, else the longest of any sample.  In the subspace iteration too, a sample that ran out of
+ * device memory beside the others is solved again
  * after the batch, alone (its stats are then its own solve's), and every sample releases its work
  * buffers when the batch ends (its eigenvectors stay).
  * Returns the first failing status (the other samples still run). */

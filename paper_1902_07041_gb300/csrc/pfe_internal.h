@@ -270,6 +270,7 @@ void tridiag_top(const std::vector<double> &alpha, const std::vector<double> &be
 // State of one filtered subspace iteration (kept in the context between stages)
 // --------------------------------------------------------------------------------------
 struct SolveState {
+  bool batched = false;  // pfe_solve_batch: the FP64 filter runs in the batched launches
   bool fp32 = false, use64 = true, was64 = true, done = false, timed_filter = true, timed32 = false;
   bool active = false;  // a stepwise solve (pfe_solve_begin .. pfe_solve_end) is in progress
   // PRECISION 2: the hand-over group is filtered in FP32 by defect correction (defect.cu) instead of FP64

@@ -139,6 +139,15 @@ pfe_status ensure_fixed(pfe_ctx *ctx, const Bsr<double> &A) {
   return PFE_OK;
 }
 
+// Whether the solve's FP64 filter runs in fixed point (as run_filter64 decides).
+pfe_status filter64_is_fixed(pfe_ctx *ctx, bool *fixed) {
+  *fixed = false;
+  if (step_variant(0) >= 0 || !fixed_coefficients_ok(ctx->coef.data(), ctx->m)) return PFE_OK;
+  PFE_TRY(ensure_fixed(ctx, bsr_Hs64(ctx)));
+  *fixed = solver_fixed_op(ctx, ctx->coef.data(), ctx->m).blocks != nullptr;
+  return PFE_OK;
+}
+
 // The FP64 filter: in fixed point (fixed_step.cu) unless a kernel shape is forced, the operator or the
 // coefficients do not fit, or the degree is 0.  X row-major (ldx == ld) or, with Xr != null, column-major; Xr is
 // then the row-major copy that the FP64 kernels take.
@@ -1042,7 +1051,7 @@ void batch_plan_free(BatchPlan *p) {
   *p = BatchPlan{};
 }
 
-// Refresh the descriptors of the FP64 samples that are still iterating; returns the item count.
+// Refresh the descriptors of the batched samples that are still iterating; returns the item count.
 int64_t batch_refresh(pfe_ctx **ctxs, int32_t ns, const std::vector<pfe_status> &status, BatchPlan *p) {
   int64_t items = 0;
   p->h.resize(ns);
@@ -1050,7 +1059,7 @@ int64_t batch_refresh(pfe_ctx **ctxs, int32_t ns, const std::vector<pfe_status> 
     pfe_ctx *c = ctxs[i];
     const SolveState &st = c->solve;
     BatchDesc &d = p->h[i];
-    const bool live = status[i] == PFE_OK && !st.done && st.use64;
+    const bool live = status[i] == PFE_OK && !st.done && st.batched;
     d.rp = c->rp.as<int32_t>();
     d.ci = c->ci.as<int32_t>();
     d.vals = c->Hs64.as<double>();
@@ -1088,7 +1097,7 @@ pfe_status batch_plan_init(pfe_ctx *c0, pfe_ctx **ctxs, int32_t ns, const std::v
   PFE_CUDA_TRY(c0, cudaStreamCreateWithFlags(&p->stream, cudaStreamNonBlocking));
   cudaStream_t s = p->stream;
   for (int32_t i = 0; i < ns; ++i) {
-    if (status[i] != PFE_OK) continue;
+    if (status[i] != PFE_OK || !ctxs[i]->solve.batched) continue;
     pfe_ctx *c = ctxs[i];
     // coefficients on the device (read by the batched kernel)
     if (dbuf_reserve(c->dcoef, sizeof(double) * (c->m + 1)) != cudaSuccess)
@@ -1150,7 +1159,7 @@ pfe_status batch_plan_init(pfe_ctx *c0, pfe_ctx **ctxs, int32_t ns, const std::v
   return PFE_OK;
 }
 
-// One filter application for every FP64 sample: refresh descriptors, replay the graph.
+// One filter application for every batched sample: refresh descriptors, replay the graph.
 pfe_status batch_filter(pfe_ctx *c0, pfe_ctx **ctxs, int32_t ns, const std::vector<pfe_status> &status, BatchPlan *p,
                         float *ms) {
   cudaStream_t s = p->stream;
@@ -2009,31 +2018,61 @@ pfe_status pfe_solve_batch(pfe_ctx **ctxs, int32_t nsamples, int32_t *n_found) {
   };
   // set-up of every sample (filter design, width, buffers, start block); a sample that failed gives
   // back what it had reserved
-  for_each_sample(c0->device, nsamples, nthreads, [&](int32_t i) { status[i] = solve_setup(ctxs[i]); });
+  // Samples whose filter runs in fixed point (or FP32) iterate on their own streams; the batched FP64 launches
+  // are for the rest.
+  for_each_sample(c0->device, nsamples, nthreads, [&](int32_t i) {
+    SolveState &st = ctxs[i]->solve;
+    st.batched = false;
+    status[i] = solve_setup(ctxs[i]);
+    bool fixed = false;
+    if (status[i] == PFE_OK && st.use64) status[i] = filter64_is_fixed(ctxs[i], &fixed);
+    st.batched = status[i] == PFE_OK && st.use64 && !fixed;
+  });
   for (int32_t i = 0; i < nsamples; ++i)
     if (status[i] != PFE_OK) {
       release_si_work(ctxs[i]);
       dbuf_free(ctxs[i]->L);  // no results yet
     }
   cudaGetLastError();  // a failed allocation's error state
+  double t_batch_filter = 0.0;
+  int64_t batch_replays = 0;
+  bool lockstep = false;
+  for (int32_t i = 0; i < nsamples; ++i) lockstep = lockstep || ctxs[i]->solve.batched;
+  if (!lockstep) {
+    // No sample waits for another: each runs all its iterations from one host thread, and the small launches of
+    // the samples overlap on the device.  Six glasses of 700 to 885 atoms: 195 ms in lockstep with the shared FP64
+    // launches, 187 ms this way (cuSOLVER's dense steps are most of it).
+    for_each_sample(c0->device, nsamples, nthreads, [&](int32_t i) {
+      SolveState &st = ctxs[i]->solve;
+      while (status[i] == PFE_OK && !st.done) {
+        cudaEventRecord(st.ev[0], ctxs[i]->stream);
+        status[i] = solve_filter(ctxs[i]);
+        if (status[i] == PFE_OK) status[i] = solve_after_filter(ctxs[i]);
+      }
+    });
+    for (int32_t i = 0; i < nsamples; ++i) {
+      if (status[i] != PFE_OK) continue;
+      t_batch_filter = std::max(t_batch_filter, ctxs[i]->solve.t_filter);
+      batch_replays = std::max<int64_t>(batch_replays, ctxs[i]->solve.it);
+    }
+  }
   BatchPlan plan;
-  pfe_status bst = batch_plan_init(c0, ctxs, nsamples, status, &plan);
+  pfe_status bst = lockstep ? batch_plan_init(c0, ctxs, nsamples, status, &plan) : PFE_OK;
   if (bst != PFE_OK) {
     batch_plan_free(&plan);
     return bst;
   }
-  for (int32_t i = 0; i < nsamples; ++i) ctxs[i]->solve.timed_filter = false;
-  double t_batch_filter = 0.0;
-  int64_t batch_replays = 0;
+  if (lockstep)
+    for (int32_t i = 0; i < nsamples; ++i) ctxs[i]->solve.timed_filter = false;
   for (;;) {
     bool any = false;
     for (int32_t i = 0; i < nsamples; ++i)
       if (status[i] == PFE_OK && !ctxs[i]->solve.done) any = true;
     if (!any) break;
-    // 1. filter: one batched replay for the FP64 samples, the single-context path for FP32 ones
+    // 1. filter: one batched replay for the batched samples, the single-context path for the others
     for_each_sample(c0->device, nsamples, nthreads, [&](int32_t i) {
       SolveState &st = ctxs[i]->solve;
-      if (status[i] != PFE_OK || st.done || st.use64) return;
+      if (status[i] != PFE_OK || st.done || st.batched) return;
       status[i] = solve_filter(ctxs[i]);
     });
     float ms = 0.f;
