@@ -744,9 +744,10 @@ StepPlan plan_steps(const Bsr<double> &A, const FixedOp &op, int32_t k, int64_t 
   StepPlan p;
   p.rank1 = A.u != nullptr;
   // Two columns a lane (16-byte gathers) once the lanes fill the GPU a few times over; before that one, for more
-  // lanes (N = 1,000, k = 16: 9.0 us a step with one, 12.0 with two; N = 5,003, k = 33: 19.8 and 20.7;
-  // N = 99,900, k = 64: 334 and 303).
-  p.cpl = aligned && k > 1 && ld % 2 == 0 && (int64_t)A.n_atoms * k >= 200000 ? 2 : 1;
+  // lanes.  us a step with one and two: N = 4,000, k = 64 19.0 and 28.5; N = 3,001, k = 100 24.1 and 33.5; N = 4,000,
+  // k = 120 30.9 and 34.3; N = 20,000, k = 26 40.9 and 37.1, k = 32 37.2 and 35.8; N = 99,900, k = 64 334 and 303;
+  // full blocks N = 3,000, k = 100 24.0 and 33.9, N = 2,500, k = 200 41.6 and 40.0.
+  p.cpl = aligned && k > 1 && ld % 2 == 0 && (int64_t)A.n_atoms * k >= 500000 ? 2 : 1;
   StepArgs &a = p.a;
   a.n_atoms = A.n_atoms;
   a.ld = ld;

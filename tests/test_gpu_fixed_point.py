@@ -249,3 +249,24 @@ def test_fixed_point_adjoint_matches_the_checkpointed_one(N, k, coef, rank1):
     finally:
         pfe.pfe_set_param(ctx, pfe.PFE_P_STEP_SHAPE_F64, -1)
         pfe.pfe_destroy(ctx)
+
+
+# two columns a lane, with an even and an odd number of columns
+@pytest.mark.parametrize("rank1", [1, 0])
+@pytest.mark.parametrize("k", [130, 131])
+def test_two_columns_a_lane(k, rank1):
+    g = glassgen.generate(4001, 22)
+    ctx = context(g, 0.25, rank1)
+    try:
+        coef = np.cos(np.arange(6)) / (1.0 + np.arange(6))
+        X = np.random.default_rng(k).standard_normal((g.n, k))
+        ref = oracle.cheb_filter(oracle.csr_from_springs(g), 0.125, 0.125, coef, X)
+        assert np.max(np.abs(apply(ctx, coef, X) - ref)) <= tolerance(X, coef)
+        Xd = torch.from_numpy(np.ascontiguousarray(X.T)).cuda()
+        rp, ci, _ = pfe.pfe_springs_to_bsr(g.n_atoms, g.bi, g.bj, g.k, g.rhat)
+        Xb, vb = torch.empty_like(Xd), torch.empty(9 * ci.size, dtype=torch.float64, device="cuda")
+        pfe.pfe_filter_adjoint(ctx, 5, coef, k, Xd, g.n, Xd, g.n, Xb, g.n, vb)  # the filter is symmetric
+        torch.cuda.synchronize()
+        assert np.max(np.abs(Xb.cpu().numpy().T - ref)) <= tolerance(X, coef)
+    finally:
+        pfe.pfe_destroy(ctx)
