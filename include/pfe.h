@@ -96,7 +96,8 @@ enum {
                                columns with the rows of the tile's neighbourhood staged in shared memory
                                (as 7 in FP64); 11: the rank-1 form as 8 compiled for six resident CTAs per
                                SM */
-  PFE_P_STEP_SHAPE_F32 = 20, /* PROCESS-WIDE: the same for the FP32 filter step */
+  PFE_P_STEP_SHAPE_F32 = 20, /* PROCESS-WIDE: the same for the FP32 filter step; -1: on the rank-1 form the step
+                               with staged blocks, reported as 13, else autotuned */
   PFE_P_METHOD = 21,        /* 0: filtered subspace iteration (Alg. 4, default); 1: thick-restart block
                                Lanczos on the filter operator (Sec. 2.5, the paper's Krylov-Schur solver),
                                FP64 only */
@@ -254,7 +255,7 @@ typedef struct {
   int32_t basis;               /* METHOD 1: maximal basis size */
   int32_t filter_shape_f64;    /* kernel shape of the last FP64 filter step (PFE_P_STEP_SHAPE_F64 numbering;
                                   7-9: the rank-1 form; 12: fixed point), -1 if none ran */
-  int32_t filter_shape_f32;    /* the same for the FP32 filter step */
+  int32_t filter_shape_f32;    /* the same for the FP32 filter step (13: staged blocks) */
   int32_t slices;              /* pfe_solve_sliced: number of slices (0 for the other solves) */
   int32_t active;              /* stepwise solve in progress: columns still iterating (0 otherwise) */
   int32_t locked;              /* stepwise solve in progress: converged pairs locked so far (0 otherwise) */

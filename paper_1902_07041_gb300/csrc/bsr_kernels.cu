@@ -314,8 +314,9 @@ bool aligned(const void *p, size_t a) { return p == nullptr || (reinterpret_cast
 // five resident CTAs; two blocks in flight); without it they fall back to shape 0.
 // A forced shape (set_step_variant) wins; otherwise the autotuner's choice for (type, columns per
 // lane, column chunks, rank-1 form present) is used, and before any tuning 7 on the rank-1 form, else 0.
-// The FP64 filter itself runs in fixed point (fixed_step.cu) unless a shape is forced; these FP64 shapes serve the
-// adjoint, products with H and operators that do not fit.
+// Unless a shape is forced the FP64 filter itself runs in fixed point (fixed_step.cu) and the FP32 filter of the
+// rank-1 form with staged blocks (r1_staged.cu); these shapes serve products with H, batches in lockstep, full FP32
+// blocks and operators that do not fit.
 namespace {
 // The tuner times the full-block shapes 0-6, or the rank-1 shapes 7-9 when the operator has that form.
 // Shape 10 (FP32, rows staged in shared memory) runs only when forced: it measured 3.6x slower than

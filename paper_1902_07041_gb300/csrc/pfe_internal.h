@@ -95,6 +95,12 @@ void launch_r1_tiled(const Bsr<float> &A, int mode, int32_t k, int64_t ld, const
 void build_r1_tiles(int32_t n_atoms, const std::vector<int32_t> &rp1, const std::vector<int32_t> &ci1,
                     std::vector<int32_t> &tile_ptr, std::vector<int32_t> &tile_atoms, std::vector<uint16_t> &slot1,
                     std::vector<uint16_t> &self_slot, int32_t *umax);
+// The FP32 filter step of the rank-1 form (r1_staged.cu), for MODE_FIRST (alpha = 1/2), MODE_STEP and MODE_STEP_ACC
+// (beta = -1); F, fs (together or neither): forcing fs[c] F of the defect-corrected filter
+bool r1_staged_usable(const Bsr<float> &A);
+void launch_r1_staged(const Bsr<float> &A, int mode, int32_t k, int64_t ld, const float *X, const float *W, float *Z,
+                      float *Y, const float *F, const float *fs, float g0, float g1, cudaStream_t s);
+constexpr int kStagedShape = 13;  // its number among the kernel shapes in pfe_stats
 // true when the autotuner chose the staged shape for FP32 steps on k columns
 bool step_prefers_tiled(int32_t k, int64_t ld);
 // true when the autotuner chose the rank-1 FP32 step at six resident CTAs per SM (shape 11) for k columns

@@ -101,6 +101,23 @@ pfe_status run_filter(pfe_ctx *ctx, const Bsr<T> &A, const double *coef, int32_t
     launch_axpby<T>(ctx->n, k, (T)coef[0], X, ld, T(0), Y, ld, s);
     return check_launch(ctx, "filter (degree 0)");
   }
+  if constexpr (sizeof(T) == 4) {
+    if (step_variant(1) < 0 && r1_staged_usable(A)) {
+      const float *prev = X;
+      float *cur = b0;
+      launch_r1_staged(A, MODE_FIRST, k, ld, X, nullptr, b0, Y, nullptr, nullptr, (T)coef[0], (T)coef[1], s);
+      for (int32_t j = 1; j < m; ++j) {
+        float *out = (prev == X) ? b1 : const_cast<T *>(prev);
+        const bool even = (j % 2) == 0, last = j == m - 1;
+        launch_r1_staged(A, even ? MODE_STEP_ACC : MODE_STEP, k, ld, cur, prev, out, (even || last) ? Y : nullptr,
+                         nullptr, nullptr, even ? (T)coef[j] : T(0), (T)coef[j + 1], s);
+        prev = cur;
+        cur = out;
+      }
+      note_step_variant(1, kStagedShape);
+      return check_launch(ctx, "filter step");
+    }
+  }
   if (tune) tune_step<T>(A, k, ld, X, b1, s);  // b1 is free until the second step
   launch_bsr_step<T>(A, MODE_FIRST, k, ld, X, nullptr, b0, Y, T(0.5), T(0), (T)coef[0], (T)coef[1], s);
   const T *tprev = X;
@@ -704,10 +721,15 @@ pfe_status solve_filter_defect(pfe_ctx *ctx, int32_t kd) {
   cudaEventRecord(st.ev32[0], s);
   const Bsr<float> A = bsr_Hs32(ctx);
   launch_defect_prep(n, act, kd, st.X, st.W, ld, st.dtheta, 1.0 / ctx->td, g[1], st.X32, st.B32a, st.R32, st.Y32, s);
-  tune_step<float>(A, act, ld, st.X32, st.B32b, s);  // B32b is free until step 1
+  const bool staged = step_variant(1) < 0 && r1_staged_usable(A);
+  if (!staged) tune_step<float>(A, act, ld, st.X32, st.B32b, s);  // B32b is free until step 1
   const bool tiled = step_prefers_tiled(act, ld) && r1_tiled_usable(A) && ld % 4 == 0;  // buffers 16-byte aligned
   const bool six = step_prefers_six_ctas(act, ld);
-  if (kp > 0)  // t_1 = A t_0 / 2 and y = g0 t_0 + g1 t_1 for the plain columns
+  // t_1 = A t_0 / 2 and y = g0 t_0 + g1 t_1 for the plain columns
+  if (kp > 0 && staged)
+    launch_r1_staged(A, MODE_FIRST, kp, ld, st.X32 + kd, nullptr, st.B32a + kd, st.Y32 + kd, nullptr, nullptr,
+                     (float)g[0], (float)g[1], s);
+  else if (kp > 0)
     launch_bsr_step<float>(A, MODE_FIRST, kp, ld, st.X32 + kd, nullptr, st.B32a + kd, st.Y32 + kd, 0.5f, 0.f,
                            (float)g[0], (float)g[1], s);
   const float *tprev = st.X32;
@@ -715,7 +737,10 @@ pfe_status solve_filter_defect(pfe_ctx *ctx, int32_t kd) {
   for (int32_t j = 1; j < m; ++j) {
     float *out = (tprev == st.X32) ? st.B32b : const_cast<float *>(tprev);
     const bool even = (j % 2) == 0, last = j == m - 1;
-    if (tiled)
+    if (staged)
+      launch_r1_staged(A, even ? MODE_STEP_ACC : MODE_STEP, act, ld, tcur, tprev, out, (even || last) ? st.Y32 : nullptr,
+                       st.R32, st.dfs + (size_t)j * ld, (float)g[j], (float)g[j + 1], s);
+    else if (tiled)
       launch_r1_tiled(A, even ? MODE_STEP_ACC : MODE_STEP, act, ld, tcur, tprev, out, (even || last) ? st.Y32 : nullptr,
                       st.R32, st.dfs + (size_t)j * ld, 1.f, -1.f, (float)g[j], (float)g[j + 1], s);
     else
@@ -726,7 +751,7 @@ pfe_status solve_filter_defect(pfe_ctx *ctx, int32_t kd) {
     tcur = out;
   }
   launch_defect_combine(n, act, st.X, ld, st.dpth, st.Y32, st.Y, s);
-  if (m > 1) note_step_variant(1, tiled ? 10 : (six ? 11 : 8));  // the forced steps: as shape 10, 11 or 8
+  if (m > 1) note_step_variant(1, staged ? kStagedShape : tiled ? 10 : six ? 11 : 8);  // the forced steps
   cudaEventRecord(st.ev32[1], s);
   st.timed32 = true;
   st.was64 = false;
