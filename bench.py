@@ -73,7 +73,12 @@ TRAFFIC = {
                                 "src": "2288ce777daee821",
                                 "bytes": 11131068288, "alg_bytes": 10086400320},
 }
-R1_SHAPES = (7, 8, 9, 10, 11)  # kernel shapes of the fused step that run on the rank-1 form
+# kernel shapes of the fused step that run on the rank-1 form (12, the fixed-point step, does on the spring
+# networks of every workload here)
+R1_SHAPES = (7, 8, 9, 10, 11, 12, 13)
+FIXED_SHAPE = 12
+# 32 x 32 + 64-bit multiply-adds a clock and SM (measured with independent chains on one GB300)
+IMAD_WIDE_RATE = 30.0
 
 
 def _src_hash(rel, begin, end):
@@ -590,6 +595,17 @@ def run_native(args, wl):
                             "filter sweeps on the launching stream",
             "filter_gbs_fp64": b_avg * st["filter_launches"] / secs64 / 1e9, "hbm_peak_gbs": hbm,
             "launches": st["filter_launches"], "operator_form": "rank1" if r1 else "bsr"}
+    if st["filter_shape_f64"] == FIXED_SHAPE:
+        # three wide integer multiply-adds for each FP64 one: 18 per off-diagonal block and column, 27 per diagonal
+        sms = torch.cuda.get_device_properties(local).multi_processor_count
+        imad = (18 * (nnzb - g.n_atoms) + 27 * g.n_atoms) * st["filter_col_steps"] / secs64 / 1e12
+        peak_imad = sms * IMAD_WIDE_RATE * sm_clock * 1e6 / 1e12
+        roof.update({"kernel": "k_fixed_step (fused Chebyshev step in 64-bit fixed point, shape 12)",
+                     "achieved": imad, "peak": peak_imad, "unit": "T wide multiply-adds/s", "frac": imad / peak_imad,
+                     "traffic": None, "fp64_equivalent_tflops": achieved,
+                     "peak_source": "SMs x 30 wide multiply-adds a clock (measured) x the median SM clock",
+                     "achieved_how": "wide integer multiply-adds of the blocks' products x column-steps / CUDA-event "
+                                     "seconds of the FP64 filter sweeps on the launching stream"})
     work_live = {"width": st["width"], "degree": st["degree"], "iterations": st["iterations"],
                  "matvecs": st["matvecs"], "active": [a for a, _ in first.profile],
                  "locked": [lk for _, lk in first.profile]}
