@@ -327,7 +327,8 @@ struct pfe_ctx {
   bool r1_32 = false;
   // the filter operator in fixed point (fixed_step.cu), built by the first FP64 filter call on it:
   // fx_kind 0 = not built, 1 = rank-1 form, 2 = full blocks, -1/-2 = that form does not fit
-  pfe::DBuf fx_blocks, fx_diag, fx_info, w_fx;
+  pfe::DBuf fx_op, w_fx;  // info (64 words), blocks, diagonal; state of the columns
+  void *fx_diag = nullptr;
   int fx_kind = 0;
   int32_t fx_max_row = 0;
   pfe::DBuf t_ptr, t_atoms, t_slot1, t_self;  // tiles of the staged FP32 step (built with the FP32 form)

@@ -143,9 +143,10 @@ pfe_status ensure_fixed(pfe_ctx *ctx, const Bsr<double> &A) {
   const int kind = A.u ? 1 : 2;
   if (std::abs(ctx->fx_kind) == kind) return PFE_OK;
   const size_t noff = (size_t)(ctx->nnzb - ctx->N), n1 = std::max<size_t>(noff, 1);
-  RESERVE(int32_t, blocks, ctx->fx_blocks, A.u ? 8 * n1 : 20 * (size_t)ctx->nnzb);
-  RESERVE(int32_t, diag, ctx->fx_diag, A.u ? 12 * (size_t)ctx->N : 4);
-  RESERVE(int32_t, info, ctx->fx_info, kFixedInfo);
+  // one allocation: allocating and freeing four took 0.1 ms of a call that builds its context (torch.autograd)
+  const size_t block_words = ((A.u ? 8 * n1 : 20 * (size_t)ctx->nnzb) + 63) / 64 * 64;
+  RESERVE(int32_t, info, ctx->fx_op, 64 + block_words + (A.u ? 12 * (size_t)ctx->N : 4));
+  int32_t *blocks = info + 64, *diag = blocks + block_words;
   launch_fixed_operator(A, blocks, diag, info, ctx->stream);
   PFE_TRY(check_launch(ctx, "fixed-point filter operator"));
   int32_t h[kFixedInfo] = {1};
@@ -153,6 +154,7 @@ pfe_status ensure_fixed(pfe_ctx *ctx, const Bsr<double> &A) {
   PFE_CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));
   ctx->fx_kind = h[0] || !fixed_row_fits(A, h[4]) ? -kind : kind;
   ctx->fx_max_row = h[4];
+  ctx->fx_diag = diag;
   return PFE_OK;
 }
 
@@ -175,7 +177,13 @@ pfe_status run_filter64(pfe_ctx *ctx, const Bsr<double> &A, const double *coef, 
     PFE_TRY(ensure_fixed(ctx, A));
     const FixedOp op = solver_fixed_op(ctx, coef, m);
     if (op.blocks) {
-      RESERVE(char, state, ctx->w_fx, fixed_state_bytes(ctx->n, k));
+      // the row-major copy's buffer is free on this path and holds the state of all but the tiniest networks
+      const size_t state_bytes = fixed_state_bytes(ctx->n, k);
+      void *state = Xr;
+      if (!Xr || (size_t)ctx->n * ld * sizeof(double) < state_bytes) {
+        RESERVE(char, own, ctx->w_fx, state_bytes);
+        state = own;
+      }
       launch_fixed_filter(A, op, coef, m, k, ld, X, ldx, Xr != nullptr, Y, b0, b1, state, s);
       note_step_variant(0, kFixedShape);
       return check_launch(ctx, "fixed-point filter");
@@ -1239,7 +1247,7 @@ pfe_status solver_filter64(pfe_ctx *ctx, int32_t k, int64_t ld, const double *X,
 FixedOp solver_fixed_op(const pfe_ctx *ctx, const double *coef, int32_t m) {
   const bool r1 = ctx->p_rank1 && ctx->r1_state == 1;
   if (ctx->fx_kind != (r1 ? 1 : 2) || step_variant(0) >= 0 || !fixed_coefficients_ok(coef, m)) return FixedOp{};
-  return FixedOp{ctx->fx_blocks.p, ctx->fx_diag.p, ctx->fx_info.as<int32_t>(), ctx->fx_max_row};
+  return FixedOp{ctx->fx_op.as<int32_t>() + 64, ctx->fx_diag, ctx->fx_op.as<int32_t>(), ctx->fx_max_row};
 }
 pfe_status solver_filter64_rows(pfe_ctx *ctx, const double *coef, int32_t m, int32_t k, int64_t ld, const double *X,
                                 double *Y, double *b0, double *b1, cudaStream_t s, bool tune) {
@@ -1441,8 +1449,7 @@ void pfe_destroy(pfe_ctx *ctx) {
                   &ctx->w_bks[0], &ctx->w_bks[1], &ctx->w_bks[2], &ctx->w_bks[3], &ctx->w_bks[4],
                   &ctx->r1_rp, &ctx->r1_ci, &ctx->r1_u64, &ctx->r1_dg64, &ctx->r1_u32, &ctx->r1_dg32,
                   &ctx->r1_flag, &ctx->w_slice[0], &ctx->w_slice[1], &ctx->w_f32e, &ctx->w_defect, &ctx->w_tau,
-                  &ctx->t_ptr, &ctx->t_atoms, &ctx->t_slot1, &ctx->t_self, &ctx->fx_blocks, &ctx->fx_diag,
-                  &ctx->fx_info, &ctx->w_fx};
+                  &ctx->t_ptr, &ctx->t_atoms, &ctx->t_slot1, &ctx->t_self, &ctx->fx_op, &ctx->w_fx};
   for (DBuf *b : bufs) dbuf_free(*b);
   for (int e = 0; e < 4; ++e)
     if (ctx->solve.ev[e]) cudaEventDestroy(ctx->solve.ev[e]);
