@@ -69,6 +69,9 @@ __device__ __forceinline__ double pow2(int e) {
   return __hiloint2double(e < -1022 ? 0 : (min(e, 1024) + 1023) << 20, 0);  // 0 and Inf outside the range
 }
 
+// the exponent clipped to [-126, 90]
+__device__ __forceinline__ float pow2f(int e) { return __int_as_float((min(max(e, -126), 90) + 127) << 23); }
+
 // Plain loads: under programmatic launch the buffers are still being written when this grid's CTAs start, so the
 // read-only path, whose data may not change during a grid's life, is not open to them.
 template <int CPL>
@@ -329,19 +332,26 @@ __global__ void __launch_bounds__(256, 3) k_fixed_step(const StepArgs a) {
     float bound = g * (float)(mj + 1);
     bool zero = mj == 0;
     if (MODE == MODE_FIRST || (MODE == MODE_ADJ && a.halved)) bound *= 0.5f;
-    if (MODE == MODE_ADJ) {
-      const int32_t my = a.ybar_mx[c], rel = shj - a.ybar_sh[c];
-      bound += fabsf((float)a.g0) * 1.001f * (float)(my + 1) * __int_as_float((min(max(rel, -126), 90) + 127) << 23);
-      zero = zero && my == 0;
-    }
     if (MODE != MODE_FIRST) {
       const int32_t mp = a.mx[sp * a.kc + c];
       q.wsh = shj - a.sh[sp * a.kc + c];
-      bound += (float)(mp + 1) * __int_as_float((min(max(q.wsh, -126), 90) + 127) << 23);
+      bound += (float)(mp + 1) * pow2f(q.wsh);
       zero = zero && mp == 0;
     }
+    // g_j Ybar can exceed a_{j+1} by any factor (g_m far below the other coefficients): its exponent `term` stays an
+    // integer, and the sum is bounded in units of 2^far where it passes the range of float
+    int far = 0;
+    if (MODE == MODE_ADJ) {
+      const int32_t my = a.ybar_mx[c];
+      if (my != 0 && a.ga.y != 0) {
+        const int term = a.ge + (shj - a.ybar_sh[c]);
+        far = max(0, term - 60);
+        bound = bound * pow2f(-far) + (float)(abs(a.ga.y) + 1) * 0x1p-29f * (float)(my + 1) * pow2f(term - far);
+      }
+      zero = zero && my == 0;
+    }
     // bound 1.001 < 2^e: room for top - kLimb - e more bits
-    const int e = ((__float_as_int(bound * 1.001f) >> 23) & 255) - 126;
+    const int e = ((__float_as_int(bound * 1.001f) >> 23) & 255) - 126 + far;
     const int room = top_of(a.info, g) - kLimb - e;
     q.o = zero ? 0 : room < 0 ? room : room > 1 ? room - 1 : 0;
     q.ysc = pow2((MODE == MODE_EMIT || MODE == MODE_ADJ ? a.emit : a.ge + 1) - (shj + q.o));

@@ -1,0 +1,82 @@
+"""The fixed-point filter and adjoint at the edges of what they take, against the FP64 kernels (a forced kernel shape).
+
+Tolerance, as in the tests of the ordinary range: 60 m^2 2^-53 max_c |x_c|_2 sum|g| bounds the rounding of both sides.
+"""
+import math
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import glassgen  # noqa: E402
+import paper_1902_07041_gb300 as pfe  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _device():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    torch.cuda.set_device(0)
+    pfe.load()
+
+
+def tolerance(X, coef):
+    m, top = len(coef) - 1, np.abs(X).max()  # the norm of X / top: the squares of very small entries are 0
+    return 60.0 * m * m * 2.0**-53 * top * np.linalg.norm(X / top, axis=0).max() * np.abs(coef).sum()
+
+
+def context(g, lmax, rank1=1):
+    rp, ci, vals = pfe.pfe_springs_to_bsr(g.n_atoms, g.bi, g.bj, g.k, g.rhat)
+    ctx = pfe.pfe_create(g.n_atoms, rp, ci, vals, g.mass)
+    pfe.pfe_set_param(ctx, pfe.PFE_P_LAMBDA_MAX, lmax)
+    pfe.pfe_set_param(ctx, pfe.PFE_P_RANK1, rank1)
+    return ctx, ci.size
+
+
+def adjoint(ctx, nnzb, coef, X, Yb, shape):
+    """Xbar and vals_bar with the automatic kernels (shape -1) or a forced shape."""
+    n, k = X.shape
+    Xd, Yd = (torch.from_numpy(np.ascontiguousarray(v.T)).cuda() for v in (X, Yb))
+    Xb, vb = torch.empty_like(Xd), torch.empty(9 * nnzb, dtype=torch.float64, device="cuda")
+    pfe.pfe_set_param(ctx, pfe.PFE_P_STEP_SHAPE_F64, shape)
+    try:
+        pfe.pfe_filter_adjoint(ctx, len(coef) - 1, np.array(coef), k, Xd, n, Yd, n, Xb, n, vb)
+        torch.cuda.synchronize()
+    finally:
+        pfe.pfe_set_param(ctx, pfe.PFE_P_STEP_SHAPE_F64, -1)
+    return Xb.cpu().numpy().T, vb.cpu().numpy()
+
+
+def heat(t, m):
+    """Chebyshev coefficients of exp(-t (1 + x)), down to the smallest numbers."""
+    def bessel(j):
+        return sum((t / 2.0) ** (2 * q + j) / (math.factorial(q) * math.factorial(q + j)) for q in range(12))
+    return [(2.0 if j else 1.0) * (-1.0) ** j * math.exp(-t) * bessel(j) for j in range(m + 1)]
+
+
+# a last coefficient far below the others, by hand and in a converged series; small ones among zeros; growing ones
+@pytest.mark.parametrize("rank1", [1, 0])
+@pytest.mark.parametrize("coef", [[0.5, 0.25, -0.3, 0.2, 1e-28], [0.5, 0.25, -0.3, 0.2, 1e-60],
+                                  [0.5, 0.25, -0.3, 0.2, 1e-280], [0.0, 0.3, 0.0, 1e-70, 0.0, 1e-200],
+                                  [1e-200, 1e-100, 1e-30, 1.0, 0.5], [1e-40, 0.5, 1e-40, 0.2, 1e-40],
+                                  heat(0.1, 60), heat(0.02, 30)])
+def test_adjoint_with_coefficients_of_very_different_size(coef, rank1):
+    g = glassgen.generate(150, 9)
+    ctx, nnzb = context(g, 0.25, rank1)
+    try:
+        rng = np.random.default_rng(5)
+        X, Yb = rng.standard_normal((g.n, 6)), rng.standard_normal((g.n, 6))
+        Yb[:, 3] *= 1e-200
+        Yb[4, 4] = np.inf
+        Yb[5, 5] = np.nan
+        (Xb, vb), (Xr, vr) = (adjoint(ctx, nnzb, coef, X, Yb, s) for s in (-1, 7 if rank1 else 0))
+        assert np.array_equal(np.isnan(Xb), np.isnan(Xr)) and np.array_equal(np.isinf(Xb), np.isinf(Xr))
+        for c in range(4):
+            assert np.max(np.abs(Xb[:, c] - Xr[:, c])) <= tolerance(Yb[:, [c]], coef), c
+        (Xb, vb), (Xr, vr) = (adjoint(ctx, nnzb, coef, X[:, :4], Yb[:, :4], s) for s in (-1, 7 if rank1 else 0))
+        assert np.max(np.abs(vb - vr)) <= 2.0 / 0.125 * 4 * tolerance(Yb[:, :4], coef) * np.linalg.norm(X, axis=0).max()
+    finally:
+        pfe.pfe_destroy(ctx)
