@@ -200,7 +200,7 @@ __device__ __forceinline__ int top_of(const int32_t *info, float g) {
   // the high limb of u . x takes |u|_1 2^(top - 30) < 2^31
   return __int_as_float(__ldg(info + 5)) < 1.9f ? by_norm : min(by_norm, 59);
 }
-// rank-1 blocks between two folds
+// rank-1 blocks between two folds (two always fit, see k_fixed_r1)
 __device__ __forceinline__ int fold_of(const int32_t *info) {
   return __int_as_float(__ldg(info + 2)) < 15.5f ? 6 : __int_as_float(__ldg(info + 3)) < 15.5f ? 4 : 2;
 }
@@ -500,9 +500,10 @@ __device__ __forceinline__ void note_row(int32_t *info, double row, bool bad) {
 }
 
 // Rank-1 form, unit 2^-60.  With |x| < 2^60 the cross terms of a row's diagonal block and F of its other blocks
-// stay below 2^59 (3 + sum |d| + sum (|u_r| + |u|_1)): info[2], info[3] get the largest such factor for F = 6, 4
-// (below 15.5: 63 bits hold them; F = 2 always does).  info[4]: the
-// longest row, info[5]: the largest |u|_1.
+// stay below 2^59 (3 + sum |d| + sum (|u_r| + |u|_1)), which 63 bits hold for a factor below 15.5: info[2], info[3]
+// get the largest one for F = 6, 4.  An operator whose factor for F = 2 is larger does not fit, nor does one with
+// |u|_1 >= 3.9 (the high limb of u . x would leave 32 bits, see top_of).  Neither occurs while the bound holds
+// (||A||_2 <= 2: |u|_2 <= sqrt(2), a diagonal row below 3.5).  info[4]: the longest row, info[5]: the largest |u|_1.
 __global__ void k_fixed_r1(int32_t n_atoms, const int32_t *__restrict__ rp1, const int32_t *__restrict__ ci1,
                            const double *__restrict__ u, const double *__restrict__ dg, int4 *blk, int2 *dgo,
                            int32_t *info) {
@@ -517,7 +518,7 @@ __global__ void k_fixed_r1(int32_t n_atoms, const int32_t *__restrict__ rp1, con
     dgo[6 * i + t] = bad ? make_int2(0, 0) : fixed_entry(-d[t], 0x1p60);
   }
   const double drow = fmax(row[0], fmax(row[1], row[2]));
-  double s6[3] = {0, 0, 0}, s4[3] = {0, 0, 0}, m6 = 0.0, m4 = 0.0, u1 = 0.0;
+  double s6[3] = {0, 0, 0}, s4[3] = {0, 0, 0}, s2[3] = {0, 0, 0}, m6 = 0.0, m4 = 0.0, m2 = 0.0, u1 = 0.0;
   const int32_t p0 = rp1[i], p1 = rp1[i + 1];
   for (int32_t p = p0; p < p1 && !bad; ++p) {
     const double v[3] = {u[3 * (int64_t)p], u[3 * (int64_t)p + 1], u[3 * (int64_t)p + 2]};
@@ -527,18 +528,21 @@ __global__ void k_fixed_r1(int32_t n_atoms, const int32_t *__restrict__ rp1, con
       break;
     }
     u1 = fmax(u1, s);
-    const bool new6 = (p - p0) % 6 == 0, new4 = (p - p0) % 4 == 0;
+    const bool new6 = (p - p0) % 6 == 0, new4 = (p - p0) % 4 == 0, new2 = (p - p0) % 2 == 0;
     for (int r = 0; r < 3; ++r) {
       row[r] += fabs(v[r]) * s;
       s6[r] = (new6 ? 0.0 : s6[r]) + fabs(v[r]) + s;
       s4[r] = (new4 ? 0.0 : s4[r]) + fabs(v[r]) + s;
+      s2[r] = (new2 ? 0.0 : s2[r]) + fabs(v[r]) + s;
       m6 = fmax(m6, s6[r]);
       m4 = fmax(m4, s4[r]);
+      m2 = fmax(m2, s2[r]);
     }
     const int2 a = fixed_entry(v[0], 0x1p60), b = fixed_entry(v[1], 0x1p60), c = fixed_entry(v[2], 0x1p60);
     blk[2 * (int64_t)p] = make_int4(a.x, a.y, b.x, b.y);
     blk[2 * (int64_t)p + 1] = make_int4(c.x, c.y, ci1[p], 0);
   }
+  bad = bad || !(u1 < 3.9 && 3.0 + drow + m2 < 15.5);
   if (!bad) {
     atomicMax(info + 2, __float_as_int((float)(3.0 + drow + m6)));
     atomicMax(info + 3, __float_as_int((float)(3.0 + drow + m4)));

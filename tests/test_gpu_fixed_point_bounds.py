@@ -80,3 +80,48 @@ def test_adjoint_with_coefficients_of_very_different_size(coef, rank1):
         assert np.max(np.abs(vb - vr)) <= 2.0 / 0.125 * 4 * tolerance(Yb[:, :4], coef) * np.linalg.norm(X, axis=0).max()
     finally:
         pfe.pfe_destroy(ctx)
+
+
+def bonds_context(n, bi, bj, k, rhat, lmax):
+    rp, ci, vals = pfe.pfe_springs_to_bsr(n, np.array(bi, np.int32), np.array(bj, np.int32), np.array(k, float),
+                                          np.array(rhat, float))
+    ctx = pfe.pfe_create(n, rp, ci, vals, np.ones(n))
+    pfe.pfe_set_param(ctx, pfe.PFE_P_LAMBDA_MAX, lmax)
+    return ctx
+
+
+def apply(ctx, coef, X, shape=-1):
+    n, k = X.shape
+    Xd = torch.from_numpy(np.ascontiguousarray(X.T)).cuda()
+    Yd = torch.full((k, n), float("nan"), device="cuda", dtype=torch.float64)
+    pfe.pfe_set_param(ctx, pfe.PFE_P_STEP_SHAPE_F64, shape)
+    try:
+        pfe.pfe_filter_apply(ctx, len(coef) - 1, np.array(coef), k, Xd, n, Yd, n, pfe.PFE_F64)
+        torch.cuda.synchronize()
+    finally:
+        pfe.pfe_set_param(ctx, pfe.PFE_P_STEP_SHAPE_F64, -1)
+    return Yd.cpu().numpy().T
+
+
+D = np.ones(3) / np.sqrt(3.0)
+
+
+# bonds along the diagonals of the axes whose u has |u|_1 = 4.2 (one bond), and two of them in a row of three atoms
+@pytest.mark.parametrize("bonds", [([0], [1], [D]), ([0, 0], [1, 2], [D, np.array([1, -1, 0]) / np.sqrt(2)])])
+def test_filter_with_a_stiff_bond_far_above_the_bound(bonds):
+    """A bound about three times below the spectrum: the operator's entries pass what the products of the fixed-point
+    form hold, and the vectors grow, in the FP64 kernels' way.  The difference is relative to the result."""
+    bi, bj, rhat = bonds
+    n, u = max(bj) + 1, 1.41 * np.sqrt(3.0)
+    k = [u * u / 4.0] + [1.4 * 1.4 * 2 / 4.0] * (len(bi) - 1)  # u_r = sqrt(4 k / bound) r
+    ctx = bonds_context(n, bi, bj, k, rhat, 1.0)
+    try:
+        rng = np.random.default_rng(1)
+        X = rng.standard_normal((3 * n, 16))
+        for m in (12, 40, 41):
+            coef = np.ones(m + 1)
+            Y, R = apply(ctx, coef, X), apply(ctx, coef, X, 7)
+            err = np.linalg.norm(Y - R, axis=0) / np.linalg.norm(R, axis=0)
+            assert err.max() <= 60.0 * m * m * 2.0**-53
+    finally:
+        pfe.pfe_destroy(ctx)
