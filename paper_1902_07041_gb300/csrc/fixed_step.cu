@@ -737,10 +737,11 @@ void launch_fixed_operator(const Bsr<double> &A, void *blocks, void *diag, int32
     PFE_LAUNCH k_fixed_full<<<grid, 128, 0, s>>>(A.n_atoms, A.rp, A.ci, A.vals, static_cast<int4 *>(blocks), info);
 }
 
+// Each coefficient by itself: a maximum by fmax would pass over a NaN.
 bool fixed_coefficients_ok(const double *coef, int32_t m) {
-  double g = 0.0;
-  for (int32_t j = 0; j <= m; ++j) g = std::fmax(g, std::fabs(coef[j]));
-  return m >= 1 && g < 0x1p60;
+  for (int32_t j = 0; j <= m; ++j)
+    if (!(std::fabs(coef[j]) < 0x1p60)) return false;
+  return m >= 1;
 }
 
 namespace {

@@ -125,3 +125,21 @@ def test_filter_with_a_stiff_bond_far_above_the_bound(bonds):
             assert err.max() <= 60.0 * m * m * 2.0**-53
     finally:
         pfe.pfe_destroy(ctx)
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+@pytest.mark.parametrize("at", [0, 2, 4])
+def test_adjoint_carries_a_non_finite_coefficient(bad, at):
+    """The adjoint does not refuse one: its results are not finite, as the FP64 kernels' are."""
+    g = glassgen.generate(100, 9)
+    ctx, nnzb = context(g, 0.25)
+    try:
+        coef = [0.5, 0.25, -0.3, 0.2, 0.1]
+        coef[at] = bad
+        rng = np.random.default_rng(5)
+        X, Yb = rng.standard_normal((g.n, 3)), rng.standard_normal((g.n, 3))
+        (Xb, vb), (Xr, vr) = (adjoint(ctx, nnzb, coef, X, Yb, s) for s in (-1, 7))
+        assert not np.isfinite(Xr).any()
+        assert np.array_equal(np.isnan(Xb), np.isnan(Xr)) and np.array_equal(np.isnan(vb), np.isnan(vr))
+    finally:
+        pfe.pfe_destroy(ctx)
