@@ -325,12 +325,17 @@ struct pfe_ctx {
   pfe::DBuf r1_rp, r1_ci, r1_u64, r1_dg64, r1_u32, r1_dg32, r1_flag;
   int r1_state = -1;
   bool r1_32 = false;
-  // the filter operator in fixed point (fixed_step.cu), built by the first FP64 filter call on it:
-  // fx_kind 0 = not built, 1 = rank-1 form, 2 = full blocks, -1/-2 = that form does not fit
-  pfe::DBuf fx_op, w_fx;  // info (64 words), blocks, diagonal; state of the columns
-  void *fx_diag = nullptr;
-  int fx_kind = 0;
-  int32_t fx_max_row = 0;
+  // The filter operator in fixed point (fixed_step.cu), built by the first FP64 filter call on it: [0] full blocks,
+  // [1] rank-1 form.  Each form has its own memory and is built once per transform (c, d), so that switching forms
+  // or building the FP32 operator leaves alone what an earlier filter on another stream may still be reading.
+  struct FixedForm {
+    pfe::DBuf op;  // info (64 words), blocks, diagonal
+    void *diag = nullptr;
+    int state = 0;  // 0 = not built, 1 = built, -1 = does not fit
+    int32_t max_row = 0;
+    double c = 0.0, d = 0.0;
+  } fx[2];
+  pfe::DBuf w_fx;  // state of the columns
   pfe::DBuf t_ptr, t_atoms, t_slot1, t_self;  // tiles of the staged FP32 step (built with the FP32 form)
   int32_t t_umax = 0;
 

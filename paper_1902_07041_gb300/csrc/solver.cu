@@ -138,23 +138,27 @@ pfe_status run_filter(pfe_ctx *ctx, const Bsr<T> &A, const double *coef, int32_t
   return check_launch(ctx, "filter step");
 }
 
-// The fixed-point form of the FP64 filter operator A, built once per operator (allocates, waits for its check).
+// The fixed-point form of the FP64 filter operator A, built once per form and transform (allocates, waits for its
+// check).
 pfe_status ensure_fixed(pfe_ctx *ctx, const Bsr<double> &A) {
-  const int kind = A.u ? 1 : 2;
-  if (std::abs(ctx->fx_kind) == kind) return PFE_OK;
+  pfe_ctx::FixedForm &f = ctx->fx[A.u ? 1 : 0];
+  if (f.state != 0 && f.c == ctx->tc && f.d == ctx->td) return PFE_OK;
+  f.state = 0;
   const size_t noff = (size_t)(ctx->nnzb - ctx->N), n1 = std::max<size_t>(noff, 1);
   // one allocation: allocating and freeing four took 0.1 ms of a call that builds its context (torch.autograd)
   const size_t block_words = ((A.u ? 8 * n1 : 20 * (size_t)ctx->nnzb) + 63) / 64 * 64;
-  RESERVE(int32_t, info, ctx->fx_op, 64 + block_words + (A.u ? 12 * (size_t)ctx->N : 4));
+  RESERVE(int32_t, info, f.op, 64 + block_words + (A.u ? 12 * (size_t)ctx->N : 4));
   int32_t *blocks = info + 64, *diag = blocks + block_words;
   launch_fixed_operator(A, blocks, diag, info, ctx->stream);
   PFE_TRY(check_launch(ctx, "fixed-point filter operator"));
   int32_t h[kFixedInfo] = {1};
   PFE_CUDA_TRY(ctx, cudaMemcpyAsync(h, info, sizeof(h), cudaMemcpyDeviceToHost, ctx->stream));
   PFE_CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));
-  ctx->fx_kind = h[0] || !fixed_row_fits(A, h[4]) ? -kind : kind;
-  ctx->fx_max_row = h[4];
-  ctx->fx_diag = diag;
+  f.state = h[0] || !fixed_row_fits(A, h[4]) ? -1 : 1;
+  f.max_row = h[4];
+  f.diag = diag;
+  f.c = ctx->tc;
+  f.d = ctx->td;
   return PFE_OK;
 }
 
@@ -318,7 +322,6 @@ pfe_status ensure_hs(pfe_ctx *ctx, bool need32) {
     RESERVE(float, p32, ctx->Hs32, (size_t)9 * ctx->nnzb);
     h32 = p32;
   }
-  ctx->fx_kind = 0;
   launch_filter_matrix(ctx->N, ctx->rp.as<int32_t>(), ctx->ci.as<int32_t>(), ctx->H.as<double>(), 2.0 / ctx->td, ctx->tc,
                        h64, h32, ctx->stream);
   PFE_TRY(check_launch(ctx, "filter matrix"));
@@ -1245,9 +1248,11 @@ pfe_status solver_filter64(pfe_ctx *ctx, int32_t k, int64_t ld, const double *X,
   return run_filter64(ctx, bsr_Hs64(ctx), ctx->coef.data(), ctx->m, k, ld, X, ld, nullptr, Y, b0, b1, ctx->stream);
 }
 FixedOp solver_fixed_op(const pfe_ctx *ctx, const double *coef, int32_t m) {
-  const bool r1 = ctx->p_rank1 && ctx->r1_state == 1;
-  if (ctx->fx_kind != (r1 ? 1 : 2) || step_variant(0) >= 0 || !fixed_coefficients_ok(coef, m)) return FixedOp{};
-  return FixedOp{ctx->fx_op.as<int32_t>() + 64, ctx->fx_diag, ctx->fx_op.as<int32_t>(), ctx->fx_max_row};
+  const pfe_ctx::FixedForm &f = ctx->fx[ctx->p_rank1 && ctx->r1_state == 1 ? 1 : 0];
+  if (f.state != 1 || f.c != ctx->tc || f.d != ctx->td || step_variant(0) >= 0 || !fixed_coefficients_ok(coef, m))
+    return FixedOp{};
+  int32_t *info = f.op.as<int32_t>();
+  return FixedOp{info + 64, f.diag, info, f.max_row};
 }
 pfe_status solver_filter64_rows(pfe_ctx *ctx, const double *coef, int32_t m, int32_t k, int64_t ld, const double *X,
                                 double *Y, double *b0, double *b1, cudaStream_t s, bool tune) {
@@ -1449,7 +1454,7 @@ void pfe_destroy(pfe_ctx *ctx) {
                   &ctx->w_bks[0], &ctx->w_bks[1], &ctx->w_bks[2], &ctx->w_bks[3], &ctx->w_bks[4],
                   &ctx->r1_rp, &ctx->r1_ci, &ctx->r1_u64, &ctx->r1_dg64, &ctx->r1_u32, &ctx->r1_dg32,
                   &ctx->r1_flag, &ctx->w_slice[0], &ctx->w_slice[1], &ctx->w_f32e, &ctx->w_defect, &ctx->w_tau,
-                  &ctx->t_ptr, &ctx->t_atoms, &ctx->t_slot1, &ctx->t_self, &ctx->fx_op, &ctx->w_fx};
+                  &ctx->t_ptr, &ctx->t_atoms, &ctx->t_slot1, &ctx->t_self, &ctx->fx[0].op, &ctx->fx[1].op, &ctx->w_fx};
   for (DBuf *b : bufs) dbuf_free(*b);
   for (int e = 0; e < 4; ++e)
     if (ctx->solve.ev[e]) cudaEventDestroy(ctx->solve.ev[e]);

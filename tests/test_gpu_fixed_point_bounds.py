@@ -143,3 +143,34 @@ def test_adjoint_carries_a_non_finite_coefficient(bad, at):
         assert np.array_equal(np.isnan(Xb), np.isnan(Xr)) and np.array_equal(np.isnan(vb), np.isnan(vr))
     finally:
         pfe.pfe_destroy(ctx)
+
+
+def test_calls_in_flight_on_another_stream_keep_their_operator():
+    """Filters on a caller's stream, queued behind one another, with calls in between that use the other form of the
+    operator or build its FP32 copy: each result is that of the same call made alone."""
+    g = glassgen.generate(8000, 3)
+    m, k, n = 150, 32, g.n
+    coef = np.cos(np.arange(m + 1.0)) / (1.0 + np.arange(m + 1.0))
+    X = torch.randn(k, n, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(4))
+    X32 = X.float()
+
+    def calls(ctx, stream, wait):
+        out = []
+        for rank1, x in ((1, X), (1, X32), (1, X), (0, X), (1, X), (0, X)):
+            pfe.pfe_set_param(ctx, pfe.PFE_P_RANK1, rank1)
+            out.append(torch.empty_like(x))
+            pfe.pfe_filter_apply(ctx, m, coef, k, x, n, out[-1], n, pfe.PFE_F32 if x is X32 else pfe.PFE_F64, stream=stream)
+            if wait:
+                torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        return out
+
+    side = torch.cuda.Stream()
+    ctxs = [context(g, 0.25)[0] for _ in range(2)]
+    try:
+        torch.cuda.synchronize()
+        alone, queued = calls(ctxs[0], side, True), calls(ctxs[1], side, False)
+        assert all(torch.equal(a, b) for a, b in zip(alone, queued))
+    finally:
+        for c in ctxs:
+            pfe.pfe_destroy(c)
