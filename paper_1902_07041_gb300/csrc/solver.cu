@@ -139,7 +139,7 @@ pfe_status run_filter(pfe_ctx *ctx, const Bsr<T> &A, const double *coef, int32_t
 }
 
 // The fixed-point form of the FP64 filter operator A, built once per form and transform (allocates, waits for its
-// check).
+// check).  Without device memory for it nothing is built, and the filter runs in the FP64 kernels.
 pfe_status ensure_fixed(pfe_ctx *ctx, const Bsr<double> &A) {
   pfe_ctx::FixedForm &f = ctx->fx[A.u ? 1 : 0];
   if (f.state != 0 && f.c == ctx->tc && f.d == ctx->td) return PFE_OK;
@@ -147,7 +147,11 @@ pfe_status ensure_fixed(pfe_ctx *ctx, const Bsr<double> &A) {
   const size_t noff = (size_t)(ctx->nnzb - ctx->N), n1 = std::max<size_t>(noff, 1);
   // one allocation: allocating and freeing four took 0.1 ms of a call that builds its context (torch.autograd)
   const size_t block_words = ((A.u ? 8 * n1 : 20 * (size_t)ctx->nnzb) + 63) / 64 * 64;
-  RESERVE(int32_t, info, f.op, 64 + block_words + (A.u ? 12 * (size_t)ctx->N : 4));
+  if (dbuf_reserve(f.op, sizeof(int32_t) * (64 + block_words + (A.u ? 12 * (size_t)ctx->N : 4))) != cudaSuccess) {
+    cudaGetLastError();  // the failed allocation's error state
+    return PFE_OK;
+  }
+  int32_t *info = f.op.as<int32_t>();
   int32_t *blocks = info + 64, *diag = blocks + block_words;
   launch_fixed_operator(A, blocks, diag, info, ctx->stream);
   PFE_TRY(check_launch(ctx, "fixed-point filter operator"));
@@ -183,14 +187,13 @@ pfe_status run_filter64(pfe_ctx *ctx, const Bsr<double> &A, const double *coef, 
     if (op.blocks) {
       // the row-major copy's buffer is free on this path and holds the state of all but the tiniest networks
       const size_t state_bytes = fixed_state_bytes(ctx->n, k);
-      void *state = Xr;
-      if (!Xr || (size_t)ctx->n * ld * sizeof(double) < state_bytes) {
-        RESERVE(char, own, ctx->w_fx, state_bytes);
-        state = own;
+      const bool in_copy = Xr && (size_t)ctx->n * ld * sizeof(double) >= state_bytes;
+      if (in_copy || dbuf_reserve(ctx->w_fx, state_bytes) == cudaSuccess) {
+        launch_fixed_filter(A, op, coef, m, k, ld, X, ldx, Xr != nullptr, Y, b0, b1, in_copy ? Xr : ctx->w_fx.p, s);
+        note_step_variant(0, kFixedShape);
+        return check_launch(ctx, "fixed-point filter");
       }
-      launch_fixed_filter(A, op, coef, m, k, ld, X, ldx, Xr != nullptr, Y, b0, b1, state, s);
-      note_step_variant(0, kFixedShape);
-      return check_launch(ctx, "fixed-point filter");
+      cudaGetLastError();  // the failed allocation's error state
     }
   }
   if (Xr) launch_colmajor_to_rowmajor<double>(ctx->n, k, X, ldx, Xr, ld, s);

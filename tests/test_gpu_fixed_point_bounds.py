@@ -174,3 +174,38 @@ def test_calls_in_flight_on_another_stream_keep_their_operator():
     finally:
         for c in ctxs:
             pfe.pfe_destroy(c)
+
+
+def test_no_room_for_the_fixed_operator():
+    """Without device memory for the fixed-point operator the filter runs in FP64, as it did."""
+    g = glassgen.generate(60000, 9)
+    ctx, nnzb = context(g, 0.25)
+    try:
+        X = torch.randn(2, g.n, dtype=torch.float64, device="cuda")
+        Y, R = torch.empty_like(X), torch.empty_like(X)
+        coef = np.array([0.5, 0.25, -0.3, 0.2, 0.1])
+        pfe.pfe_set_param(ctx, pfe.PFE_P_STEP_SHAPE_F64, 7)
+        pfe.pfe_filter_apply(ctx, 4, coef, 2, X, g.n, R, g.n, pfe.PFE_F64)  # builds the operator, reserves the buffers
+        pfe.pfe_set_param(ctx, pfe.PFE_P_STEP_SHAPE_F64, -1)
+        torch.cuda.synchronize()
+        hold = []
+        size = 1 << 36
+        while size >= 1 << 22:
+            try:
+                hold.append(torch.empty(size, dtype=torch.uint8, device="cuda"))
+            except torch.OutOfMemoryError:
+                size >>= 1
+        try:
+            pfe.pfe_filter_apply(ctx, 4, coef, 2, X, g.n, Y, g.n, pfe.PFE_F64)
+            torch.cuda.synchronize()
+        finally:
+            del hold
+            torch.cuda.empty_cache()
+        assert (Y - R).abs().max() <= tolerance(X.cpu().numpy().T, coef)
+        pfe.pfe_filter_apply(ctx, 4, coef, 2, X, g.n, Y, g.n, pfe.PFE_F64)  # with the memory back: in fixed point
+        torch.cuda.synchronize()
+        assert not torch.equal(Y, R)
+        assert (Y - R).abs().max() <= tolerance(X.cpu().numpy().T, coef)
+    finally:
+        pfe.pfe_set_param(ctx, pfe.PFE_P_STEP_SHAPE_F64, -1)
+        pfe.pfe_destroy(ctx)
