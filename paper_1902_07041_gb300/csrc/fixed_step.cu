@@ -23,8 +23,10 @@
 // concentrated on few atoms) move their exponent.  M of the new vector is an atomic maximum that starts at 1/16
 // of a recent one, so that few lanes write.  State: 4 rotating slots of sh and M per column.
 //
-// Columns with an Inf, a NaN or entries beyond 2^+-900 keep doubles in the same buffers and take the FP64 FMAs
-// inside the same kernel (kRaw), so every input gives what it gave before.
+// Columns with an Inf, a NaN or a largest entry beyond 2^+-800 keep doubles in the same buffers and take the FP64 FMAs
+// inside the same kernel (kRaw), so every input gives what it gave before.  With the largest coefficient between
+// 2^-100 and 2^60 one unit of the result, 2^-60 of the column's largest term, is then a normal double.
+#include <algorithm>
 #include <cmath>
 
 #include "pfe_internal.h"
@@ -629,7 +631,7 @@ __global__ void k_fixed_plan(int32_t k, int32_t parts, const uint64_t *__restric
     for (int32_t q = 0; q < parts; ++q) m = max(m, part[(int64_t)q * k + c]);
     if (m == 0) continue;
     const double v = __longlong_as_double((long long)m);
-    if (!(v >= 0x1p-900 && v <= 0x1p900)) {
+    if (!(v >= 0x1p-800 && v <= 0x1p800)) {
       raw = true;
       continue;
     }
@@ -739,9 +741,12 @@ void launch_fixed_operator(const Bsr<double> &A, void *blocks, void *diag, int32
 
 // Each coefficient by itself: a maximum by fmax would pass over a NaN.
 bool fixed_coefficients_ok(const double *coef, int32_t m) {
-  for (int32_t j = 0; j <= m; ++j)
+  double g = 0.0;
+  for (int32_t j = 0; j <= m; ++j) {
     if (!(std::fabs(coef[j]) < 0x1p60)) return false;
-  return m >= 1;
+    g = std::max(g, std::fabs(coef[j]));
+  }
+  return m >= 1 && g >= 0x1p-100;
 }
 
 namespace {

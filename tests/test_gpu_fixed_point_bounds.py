@@ -209,3 +209,21 @@ def test_no_room_for_the_fixed_operator():
     finally:
         pfe.pfe_set_param(ctx, pfe.PFE_P_STEP_SHAPE_F64, -1)
         pfe.pfe_destroy(ctx)
+
+
+@pytest.mark.parametrize("x,g", [(1e-260, 1e-40), (1e-230, 1e-60), (1.0, 1e-300), (1e-200, 1e-90)])
+def test_filter_and_adjoint_keep_tiny_results(x, g):
+    net = glassgen.generate(100, 9)
+    ctx, nnzb = context(net, 0.25)
+    try:
+        coef = g * np.array([0.5, 0.25, -0.3, 0.2, 0.1])
+        rng = np.random.default_rng(5)
+        X, Yb = rng.standard_normal((net.n, 3)), x * rng.standard_normal((net.n, 3))
+        Y, R = apply(ctx, coef, Yb), apply(ctx, coef, Yb, 7)
+        assert np.abs(R).max() > 0
+        (Xb, vb), (Xr, vr) = (adjoint(ctx, nnzb, coef, X, Yb, s) for s in (-1, 7))
+        assert np.abs(Y - R).max() <= 1e-12 * np.abs(R).max()
+        assert np.abs(Xb - Xr).max() <= 1e-12 * np.abs(Xr).max()
+        assert np.abs(vb - vr).max() <= 1e-11 * np.abs(vr).max()
+    finally:
+        pfe.pfe_destroy(ctx)
