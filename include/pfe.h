@@ -286,7 +286,10 @@ pfe_status pfe_filter_apply(pfe_ctx *ctx, int32_t m, const double *coeffs, int32
 /* Adjoint of Y = p_m(Ht) X for L = <Ybar, Y> with c, d held fixed (FP64 only):
  *   Xbar = p_m(Ht)^T Ybar = p_m(Ht) Ybar,
  *   vals_bar[9 nnzb] = dL/dH for each stored entry of H (same layout as vals).
- * The recurrence is recomputed from about sqrt(m) stored checkpoints of (t_j, t_{j-1}).
+ * The context keeps the vectors t_j and a_j of the sweep, about 2 m blocks of n x k doubles, while they take at most
+ * a 64th of the device's memory and an eighth of what is free when the buffer grows; beyond that the recurrence runs in
+ * segments, down to sqrt(m) steps, whose vectors are recomputed from saved pairs (t_j, t_{j-1}): about 4 sqrt(m)
+ * blocks.  The buffer stays with the context until pfe_destroy.
  * All arrays are DEVICE pointers; X, Ybar, Xbar column-major n x k.  vals_bar is overwritten. */
 pfe_status pfe_filter_adjoint(pfe_ctx *ctx, int32_t m, const double *coeffs, int32_t k, const double *X,
                               int64_t ldx, const double *Ybar, int64_t ldyb, double *Xbar, int64_t ldxb,

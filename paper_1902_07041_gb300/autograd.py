@@ -3,7 +3,7 @@
 The forward pass assembles Delta from the spring constants (eq. (1)), forms H = M^-1/2 Delta M^-1/2
 (eq. (2)) and applies Alg. 2 through pfe_filter_apply.  The backward pass calls pfe_filter_adjoint
 (X_bar = p(Ht) Y_bar, and dL/dH per stored entry from the reverse sweep of the three-term recurrence,
-recomputed from about sqrt(m) checkpoints) and pfe_chain_springs (dL/dk per bond, dL/dm per atom).
+whose vectors are kept while they take little of the device's memory, else recomputed in segments) and pfe_chain_springs (dL/dk per bond, dL/dm per atom).
 The spectral transform Ht = (H - cI)/d is held fixed: c and d come from the given lambda bounds,
 they are not differentiated.
 

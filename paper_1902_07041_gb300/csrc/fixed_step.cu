@@ -898,67 +898,133 @@ void launch_fixed_filter(const Bsr<double> &A, const FixedOp &op, const double *
   }
 }
 
-size_t fixed_adjoint_state_bytes(int64_t n, int32_t k) {
-  return fixed_state_bytes(n, k) + (size_t)(4 * ((k + 3) / 4 * 4)) * sizeof(int32_t);
+namespace {
+
+__global__ void k_copy16(int64_t words, const int4 *__restrict__ a, int4 *__restrict__ b) {
+  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < words; t += (int64_t)gridDim.x * blockDim.x) b[t] = a[t];
+}
+void copy16(const void *a, void *b, int64_t words, cudaStream_t s) {
+  PFE_LAUNCH k_copy16<<<(unsigned)std::min<int64_t>((words + 255) / 256, 4096), 256, 0, s>>>(
+      words, static_cast<const int4 *>(a), static_cast<int4 *>(b));
+}
+int32_t segments(int32_t m, int32_t seg) { return (m + seg - 1) / seg; }
+int32_t snapshots(int32_t m, int32_t seg) { return std::max(0, segments(m, seg) - 2); }
+
+}  // namespace
+
+// Segments of `seg` steps: Ybar as it came and in fixed point, a_j and a_{j+1}, the segment's t_j and a_j; with more
+// than one segment also the forward pair and a saved pair for each segment but the first and the last
+int64_t fixed_adjoint_vectors(int32_t m, int32_t seg) {
+  return 4 + 2 * (int64_t)seg + 1 + (segments(m, seg) > 1 ? 2 : 0) + 2 * (int64_t)snapshots(m, seg);
+}
+size_t fixed_adjoint_state_bytes(int64_t n, int32_t k, int32_t m, int32_t seg) {
+  const int64_t kc = (k + 3) / 4 * 4;
+  return fixed_state_bytes(n, k) + (size_t)((12 + 8 * snapshots(m, seg)) * kc) * sizeof(int32_t);
 }
 
-void launch_fixed_adjoint(const Bsr<double> &A, const FixedOp &op, const double *coef, int32_t m, int32_t k, int64_t ld,
-                          const double *Ybar, double *t, double *adj, double *b0, double *b1, double *b2, void *state,
-                          cudaStream_t s) {
+// One segment keeps every t_j and a_j: 2 m steps.  More recompute the t_j of each from a saved pair (with its exponents,
+// so that they are the same bits), up to 3 m steps: N = 20,000, k = 32, m = 60 takes 14.7 ms with one segment.
+const double *launch_fixed_adjoint(const Bsr<double> &A, const FixedOp &op, const double *coef, int32_t m, int32_t seg,
+                                   int32_t k, int64_t ld, const double *X, int64_t ldx, const double *Ybar, int64_t ldyb,
+                                   int64_t nnzb, double two_over_d, double *vals_bar, double *work, void *state,
+                                   cudaStream_t s) {
   const int64_t n = 3 * (int64_t)A.n_atoms, vec = n * ld;
-  StepPlan p = plan_steps(A, op, k, ld, aligned16(t) && aligned16(adj) && aligned16(b0) && aligned16(b1) && aligned16(b2) && vec % 2 == 0);
+  StepPlan p = plan_steps(A, op, k, ld, aligned16(work) && vec % 2 == 0);
   StepArgs &a = p.a;
-  a.sh = static_cast<int32_t *>(state);
-  a.mx = a.sh + 4 * a.kc;
-  int32_t *ysh = a.mx + 4 * a.kc, *ymx = ysh + 2 * a.kc;
-  uint64_t *part = reinterpret_cast<uint64_t *>(ymx + 2 * a.kc);
-  int2 *v0 = reinterpret_cast<int2 *>(b0), *v1 = reinterpret_cast<int2 *>(b1), *yb = reinterpret_cast<int2 *>(b2);
-  // t_1 .. t_{m-1}
-  if (m > 1) {
-    plan_columns(p, n, k, t, ld, false, a.sh, a.mx, part, s);
-    convert_columns(p, n, k, t, ld, false, a.sh, v0, s);
-    for (int32_t j = 0; j + 1 < m; ++j) {
-      a.j = j;
-      a.X = j % 2 == 0 ? v0 : v1;
-      a.W = a.Z = j % 2 == 0 ? v1 : v0;
-      a.Y = t + (j + 1) * vec;
-      a.emit = 0;
-      a.ge = 1;  // MODE_FIRST: y = 0 x + 1 t_1
-      a.ga = make_int2(0, 0);
-      a.gb = fixed_coefficient(1.0, 1);
-      a.g0 = 0.0;
-      a.g1 = 1.0;
-      launch_planned(p, j == 0 ? MODE_FIRST : MODE_EMIT, s);
-    }
-  }
-  // a_{m-1} .. a_0 from a_m = g_m Ybar; the coefficients scaled to at most 1 so that tiny ones keep their accuracy
+  const int32_t nseg = segments(m, seg), saved = snapshots(m, seg);
+  const int64_t kc = a.kc;
+  int32_t *ash = static_cast<int32_t *>(state), *amx = ash + 4 * kc, *ysh = ash + 8 * kc, *ymx = ysh + 2 * kc;
+  int32_t *fsh = ash + 12 * kc, *fmx = fsh + 4 * kc, *save_state = fsh + 8 * kc;
+  uint64_t *part = reinterpret_cast<uint64_t *>(save_state + 8 * saved * kc);
+  double *t = work, *adj = t + seg * vec, *yr = adj + (seg + 1) * vec;
+  int2 *yb = reinterpret_cast<int2 *>(yr + vec), *v0 = yb + vec, *v1 = v0 + vec;
+  int2 *f0 = nseg > 1 ? v1 + vec : v0, *f1 = f0 + vec, *save = f1 + vec;  // save: unused with fewer than three segments
+  launch_colmajor_to_rowmajor<double>(n, k, Ybar, ldyb, yr, ld, s);
+
+  const auto start = [&] {  // t_0 in t and, in fixed point, in f0
+    launch_colmajor_to_rowmajor<double>(n, k, X, ldx, t, ld, s);
+    if (m == 1) return;
+    plan_columns(p, n, k, t, ld, false, fsh, fmx, part, s);
+    convert_columns(p, n, k, t, ld, false, fsh, f0, s);
+  };
+  const auto forward = [&](int32_t j, double *out) {  // t_{j+1} from t_j, t_{j-1}; out (never null for j = 0): in FP64
+    a.sh = fsh;
+    a.mx = fmx;
+    a.j = j;
+    a.X = j % 2 == 0 ? f0 : f1;
+    a.W = a.Z = j % 2 == 0 ? f1 : f0;
+    a.Y = out;
+    a.emit = 0;
+    a.halved = 0;
+    a.ge = 1;  // MODE_FIRST: y = 0 x + 1 t_1
+    a.ga = make_int2(0, 0);
+    a.gb = fixed_coefficient(1.0, 1);
+    a.g0 = 0.0;
+    a.g1 = 1.0;
+    launch_planned(p, j == 0 ? MODE_FIRST : out ? MODE_EMIT : MODE_STEP, s);
+  };
+  // the coefficients scaled to at most 1 so that tiny ones keep their accuracy
   double top = 0.0;
   for (int32_t j = 0; j <= m; ++j) top = std::fmax(top, std::fabs(coef[j]));
   const int up = coefficient_exponent(top);
-  launch_axpby<double>(n, k, std::ldexp(coef[m], -up), Ybar, ld, 0.0, adj + m * vec, ld, s);
-  plan_columns(p, n, k, Ybar, ld, false, ysh, ymx, part, s);
-  plan_columns(p, n, k, adj + m * vec, ld, false, a.sh, a.mx, part, s);
-  PFE_LAUNCH k_fixed_adjoint_columns<<<(unsigned)((a.kc / p.cpl + 127) / 128), 128, 0, s>>>(a.kc, p.cpl, a.sh, a.mx, ysh, ymx);
-  convert_columns(p, n, k, Ybar, ld, false, ysh, yb, s);
-  convert_columns(p, n, k, adj + m * vec, ld, false, a.sh, v0, s);
-  cudaMemsetAsync(v1, 0, (size_t)vec * sizeof(int2), s);
-  launch_axpby<double>(n, k, coef[m], Ybar, ld, 0.0, adj + m * vec, ld, s);
-  a.Ybar = yb;
-  a.ybar_sh = ysh;
-  a.ybar_mx = ymx;
-  a.emit = up;
-  for (int32_t r = 0; r < m; ++r) {
-    const int32_t j = m - 1 - r;
+  const auto reverse_start = [&](double *am) {  // a_m = g_m Ybar in am and, in fixed point, in v0; a_{m+1} = 0 in v1
+    launch_axpby<double>(n, k, std::ldexp(coef[m], -up), yr, ld, 0.0, am, ld, s);
+    plan_columns(p, n, k, yr, ld, false, ysh, ymx, part, s);
+    plan_columns(p, n, k, am, ld, false, ash, amx, part, s);
+    PFE_LAUNCH k_fixed_adjoint_columns<<<(unsigned)((kc / p.cpl + 127) / 128), 128, 0, s>>>(kc, p.cpl, ash, amx, ysh, ymx);
+    convert_columns(p, n, k, yr, ld, false, ysh, yb, s);
+    convert_columns(p, n, k, am, ld, false, ash, v0, s);
+    cudaMemsetAsync(v1, 0, (size_t)vec * sizeof(int2), s);
+    launch_axpby<double>(n, k, coef[m], yr, ld, 0.0, am, ld, s);
+  };
+  const auto reverse = [&](int32_t j, double *out) {  // a_j from a_{j+1}, a_{j+2}
+    const int32_t r = m - 1 - j;
+    a.sh = ash;
+    a.mx = amx;
     a.j = r;
     a.X = r % 2 == 0 ? v0 : v1;
     a.W = a.Z = r % 2 == 0 ? v1 : v0;
-    a.Y = adj + j * vec;
+    a.Y = out;
+    a.Ybar = yb;
+    a.ybar_sh = ysh;
+    a.ybar_mx = ymx;
+    a.emit = up;
     a.halved = j == 0;
     a.g0 = std::ldexp(coef[j], -up);
     a.ge = coefficient_exponent(a.g0);
     a.ga = fixed_coefficient(a.g0, a.ge);
     launch_planned(p, MODE_ADJ, s);
+  };
+
+  // The step that gives segment g's first vector t_{g seg} is step g seg - 1: the state before it is saved, and stays
+  // in f0, f1 for the last segment.
+  if (nseg > 1) {
+    start();
+    for (int32_t j = 0; j < (nseg - 1) * seg - 1; ++j) {
+      const int32_t g = (j + 1) / seg;
+      if ((j + 1) % seg == 0 && g <= saved) {
+        copy16(f0, save + 2 * (g - 1) * vec, vec, s);  // f0 and f1
+        copy16(fsh, save_state + 8 * (g - 1) * kc, 2 * kc, s);
+      }
+      forward(j, j == 0 ? adj : nullptr);
+    }
   }
+  for (int32_t g = nseg - 1; g >= 0; --g) {
+    const int32_t j0 = g * seg, j1 = std::min(m, j0 + seg);
+    if (g == 0) {
+      start();
+    } else if (g < nseg - 1) {
+      copy16(save + 2 * (g - 1) * vec, f0, vec, s);
+      copy16(save_state + 8 * (g - 1) * kc, fsh, 2 * kc, s);
+    }
+    for (int32_t j = std::max(0, j0 - 1); j + 1 < j1; ++j) forward(j, t + (j + 1 - j0) * vec);
+    if (g == nseg - 1) reverse_start(adj + (j1 - j0) * vec);
+    else copy16(adj, adj + seg * vec, vec / 2, s);  // a_{j1}
+    for (int32_t j = j1 - 1; j >= j0; --j) reverse(j, adj + (j - j0) * vec);
+    launch_outer_accum_seg(A, nnzb, k, ld, j1 - j0, vec, adj + vec, t, two_over_d * (g == 0 ? 0.5 : 1.0), two_over_d,
+                           vals_bar, s);
+  }
+  return adj;
 }
 
 }  // namespace pfe

@@ -178,12 +178,15 @@ bool fixed_coefficients_ok(const double *coef, int32_t m);
 void launch_fixed_filter(const Bsr<double> &A, const FixedOp &op, const double *coef, int32_t m, int32_t k, int64_t ld,
                          const double *X, int64_t ldx, bool colmajor, double *Y, double *b0, double *b1, void *state,
                          cudaStream_t s);
-// The adjoint's recurrences: t holds t_0 and receives t_1 .. t_{m-1}, adj receives a_0 .. a_m (vectors of n x ld
-// doubles one after another); b0, b1, b2: one such vector each, state: fixed_adjoint_state_bytes(n, k); m >= 1
-size_t fixed_adjoint_state_bytes(int64_t n, int32_t k);
-void launch_fixed_adjoint(const Bsr<double> &A, const FixedOp &op, const double *coef, int32_t m, int32_t k, int64_t ld,
-                          const double *Ybar, double *t, double *adj, double *b0, double *b1, double *b2, void *state,
-                          cudaStream_t s);
+// The adjoint in segments of `seg` of the m >= 1 steps (seg = m: nothing is recomputed); X, Ybar column-major.  Adds
+// the outer products to vals_bar and returns Xbar (row-major n x ld, in work).  work: fixed_adjoint_vectors(m, seg)
+// vectors of n x ld doubles, state: fixed_adjoint_state_bytes
+int64_t fixed_adjoint_vectors(int32_t m, int32_t seg);
+size_t fixed_adjoint_state_bytes(int64_t n, int32_t k, int32_t m, int32_t seg);
+const double *launch_fixed_adjoint(const Bsr<double> &A, const FixedOp &op, const double *coef, int32_t m, int32_t seg,
+                                   int32_t k, int64_t ld, const double *X, int64_t ldx, const double *Ybar, int64_t ldyb,
+                                   int64_t nnzb, double two_over_d, double *vals_bar, double *work, void *state,
+                                   cudaStream_t s);
 constexpr int kFixedShape = 12;  // its number among the kernel shapes in pfe_stats
 
 // Batched filter: one persistent launch per Chebyshev step over every sample's work items.

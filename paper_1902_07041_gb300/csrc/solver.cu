@@ -1865,21 +1865,35 @@ pfe_status pfe_filter_adjoint(pfe_ctx *ctx, int32_t m, const double *coeffs, int
   const size_t vec = (size_t)n * ld;
   const Bsr<double> A = bsr_Hs64(ctx);
   const double two_over_d = 2.0 / ctx->td;
-  // In fixed point with every t_j and a_j kept (no recomputation) while they take at most 16 GB; a device without
-  // that room, an operator that does not fit and larger problems take the checkpoints below.
-  if (m >= 1 && step_variant(0) < 0 && fixed_coefficients_ok(cf, m) && (2 * (size_t)m + 6) * vec * sizeof(double) <= ((size_t)16 << 30)) {
+  // In fixed point; an operator that does not fit, and a device without room, take the FP64 kernels below.
+  if (m >= 1 && step_variant(0) < 0 && fixed_coefficients_ok(cf, m)) {
     PFE_TRY(ensure_fixed(ctx, A));
     const FixedOp op = solver_fixed_op(ctx, cf, m);
-    const size_t state_bytes = (fixed_adjoint_state_bytes(n, k) + 255) / 256 * 256;
-    if (op.blocks && dbuf_reserve(ctx->w_ckpt, state_bytes + (2 * (size_t)m + 6) * vec * sizeof(double)) == cudaSuccess) {
-      void *state = ctx->w_ckpt.p;
-      double *t = reinterpret_cast<double *>(static_cast<char *>(state) + state_bytes), *adj = t + (size_t)m * vec;
-      double *Yb = adj + ((size_t)m + 1) * vec, *b0 = Yb + vec, *b1 = b0 + vec, *b2 = b1 + vec;
-      launch_colmajor_to_rowmajor<double>(n, k, X, ldx, t, ld, s);
-      launch_colmajor_to_rowmajor<double>(n, k, Ybar, ldyb, Yb, ld, s);
-      launch_fixed_adjoint(A, op, cf, m, k, ld, Yb, t, adj, b0, b1, b2, state, s);
-      launch_outer_accum_seg(A, ctx->nnzb, k, ld, m, (int64_t)vec, adj + vec, t, 0.5 * two_over_d, two_over_d, vals_bar, s);
-      launch_rowmajor_to_colmajor<double>(n, k, adj, ld, Xbar, ldxb, s);
+    const auto state_bytes = [&](int32_t seg) { return (fixed_adjoint_state_bytes(n, k, m, seg) + 255) / 256 * 256; };
+    const auto bytes = [&](int32_t seg) {
+      return state_bytes(seg) + (size_t)fixed_adjoint_vectors(m, seg) * vec * sizeof(double);
+    };
+    // Segments as long as the memory allows: all steps in one while that takes at most a 64th of the device (4.4 GB
+    // of 280; the context keeps the buffer) and an eighth of what is free, else down to sqrt(m) steps, the least
+    // memory.  Below 64 MB nothing is asked: the query would cost short calls more than the memory matters.
+    const int32_t least = (int32_t)std::ceil(std::sqrt((double)m));
+    int32_t seg = m;
+    if (op.blocks && bytes(m) > std::max(ctx->w_ckpt.bytes, (size_t)64 << 20)) {
+      size_t free_bytes = 0, total = 0;
+      if (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess) cudaGetLastError();
+      const size_t limit = std::max(ctx->w_ckpt.bytes, std::min(total / 64, (free_bytes + ctx->w_ckpt.bytes) / 8));
+      for (int32_t g = 2; seg > least && bytes(seg) > limit; ++g) seg = std::max(least, (m + g - 1) / g);
+    }
+    bool room = op.blocks && dbuf_reserve(ctx->w_ckpt, bytes(seg)) == cudaSuccess;
+    if (op.blocks && !room && seg > least) {
+      seg = least;
+      room = dbuf_reserve(ctx->w_ckpt, bytes(seg)) == cudaSuccess;
+    }
+    if (room) {
+      double *work = reinterpret_cast<double *>(static_cast<char *>(ctx->w_ckpt.p) + state_bytes(seg));
+      const double *a0 = launch_fixed_adjoint(A, op, cf, m, seg, k, ld, X, ldx, Ybar, ldyb, ctx->nnzb, two_over_d, vals_bar,
+                                              work, ctx->w_ckpt.p, s);
+      launch_rowmajor_to_colmajor<double>(n, k, a0, ld, Xbar, ldxb, s);
       return check_launch(ctx, "filter_adjoint");
     }
     cudaGetLastError();  // a failed allocation's error state

@@ -227,3 +227,65 @@ def test_filter_and_adjoint_keep_tiny_results(x, g):
         assert np.abs(vb - vr).max() <= 1e-11 * np.abs(vr).max()
     finally:
         pfe.pfe_destroy(ctx)
+
+
+def device_adjoint(ctx, nnzb, coef, X, Yb):
+    k, n = X.shape
+    Xb, vb = torch.empty_like(X), torch.empty(9 * nnzb, dtype=torch.float64, device="cuda")
+    pfe.pfe_filter_adjoint(ctx, len(coef) - 1, coef, k, X, n, Yb, n, Xb, n, vb)
+    torch.cuda.synchronize()
+    return Xb, vb
+
+
+def test_adjoint_keeps_at_most_a_64th_of_the_device():
+    """200 steps of 64 columns keep 12 GB of vectors: more than a 64th of the device, so they are run in segments."""
+    g = glassgen.generate(20000, 9)
+    ctx, nnzb = context(g, 0.25)
+    try:
+        k, m = 64, 200
+        gen = torch.Generator("cuda").manual_seed(6)
+        X, Yb = (torch.randn(k, g.n, dtype=torch.float64, device="cuda", generator=gen) for _ in range(2))
+        coef = np.cos(np.arange(m + 1.0)) / (1.0 + np.arange(m + 1.0))
+        torch.cuda.synchronize()
+        free, total = torch.cuda.mem_get_info()
+        Xb, vb = device_adjoint(ctx, nnzb, coef, X, Yb)
+        taken = free - torch.cuda.mem_get_info()[0]
+        assert taken <= total / 64 + 2**29  # and the operator, Xbar and the gradient
+        pfe.pfe_set_param(ctx, pfe.PFE_P_STEP_SHAPE_F64, 7)
+        Xr, vr = device_adjoint(ctx, nnzb, coef, X, Yb)
+        tol = tolerance(Yb.cpu().numpy().T, coef)
+        assert (Xb - Xr).abs().max() <= tol
+        assert (vb - vr).abs().max() <= 2.0 / 0.125 * k * tol * X.norm(dim=1).max().item()
+    finally:
+        pfe.pfe_set_param(ctx, pfe.PFE_P_STEP_SHAPE_F64, -1)
+        pfe.pfe_destroy(ctx)
+
+
+# segments of one step to several, a short last one, one saved pair to many
+@pytest.mark.parametrize("rank1", [1, 0])
+@pytest.mark.parametrize("m", [2, 3, 5, 10, 30])
+def test_adjoint_in_segments_gives_the_bits_of_one_segment(m, rank1):
+    """On a device nearly full the vectors are recomputed from saved pairs: the same vectors, so the same Xbar."""
+    g = glassgen.generate(8000, 9)
+    ctxs = [context(g, 0.25, rank1) for _ in range(2)]
+    hold = None
+    try:
+        k = 63
+        gen = torch.Generator("cuda").manual_seed(6)
+        X, Yb = (torch.randn(k, g.n, dtype=torch.float64, device="cuda", generator=gen) for _ in range(2))
+        X[5] *= 1e-290  # kept in FP64
+        coef = np.cos(np.arange(m + 1.0)) / (1.0 + np.arange(m + 1.0))
+        ref = device_adjoint(*ctxs[0], coef, X, Yb)
+        small = device_adjoint(*ctxs[1], coef[:2], X[:1], Yb[:1])  # the operator is built
+        torch.cuda.empty_cache()
+        least = int(np.ceil(np.sqrt(m)))
+        room = 8 * g.n * 64 * (2 * least + 2 * -(-m // least) + 5) + 2**27
+        hold = torch.empty(torch.cuda.mem_get_info()[0] - room, dtype=torch.uint8, device="cuda")
+        got = device_adjoint(*ctxs[1], coef, X, Yb)
+        assert small[0].isfinite().all() and torch.equal(got[0], ref[0])
+        assert (got[1] - ref[1]).abs().max() <= 1e-13 * ref[1].abs().max()  # sums over segments in another order
+    finally:
+        del hold
+        torch.cuda.empty_cache()
+        for c, _ in ctxs:
+            pfe.pfe_destroy(c)
