@@ -3,13 +3,22 @@
 // Why: the Gram matrices and block updates of the solvers are n x q x q products.  GB300's FP64 tensor path runs at
 // 1.1 TFLOP/s, tcgen05 at 1,900 in BF16.  Every operand entry becomes seven signed 8-bit digits (55 bits below the
 // largest entry of its row or column); BF16 holds a digit, and FP32 a sum of 1,024 digit products, exactly.  The 28
-// products of digits i + j <= 6 are exact up to integer sums, so the only errors are the dropped low digits, 2^-56 of
-// the largest entries: below the rounding of an FP64 sum.
+// products of digits i + j <= 6 are summed exactly, the six of i + j = 7 in FP32, so an entry C_pq is off by at most
+//   2^-56 (e_p |b_q|_1 + e_q |a_p|_1) + K 2^-61 e_p e_q,   e: the power of two above the largest entry,
+// from the digits below the 55th bit and the products of i + j >= 8.  Measured against exact sums, unit columns:
+// normal entries 2e-16 (the FP64 tensor path 8e-16); columns localised on one of 300,000 rows 5.4e-15 on the diagonal
+// (1.3e-15 to 4e-15; at 3,000 rows 2e-16 and 2e-15), as the squares of a column's fifth digits all add up, and 6e-17 off
+// it.  With i + j <= 6 alone (28 products) those were 1.6e-14 and 1e-14; the 34 take 1.2 times as long (300,000 x 994:
+// Gram 13.5 -> 16.3 ms, update 26.6 -> 32.5; on the FP64 tensor path 341 and 563).
+// All this is relative to the columns' largest entries: an entry of C that sums small products only (columns whose
+// large entries lie in different rows) keeps fewer digits than in FP64.
 //
-// Sums.  The digit products of equal weight i + j = g share one TMEM accumulator (128 x 64 FP32, seven of them:
-// 448 of 512 columns).  After 128 terms (7 x 128 x 2^14 < 2^24) the epilogue warps add them as integers into two
-// 64-bit sums a tile element, hi (g = 0..2) and lo (g = 3..6), value hi 2^32 + lo.  Splitting the contraction over
-// CTAs therefore gives the same bits in any order.
+// Sums.  The digit products of equal weight i + j = g share one TMEM accumulator (128 x 64 FP32, eight of them: all
+// 512 columns).  After 128 terms (7 x 128 x 2^14 < 2^24) the epilogue warps add them as integers into two 64-bit sums
+// a tile element, hi (g = 0..3) and lo (g = 4..7), value hi 2^32 + lo.  The last weight, g = 7, needs no exact sum (its
+// rounding in FP32 is 2^-23 of 2^-53): it stays in its accumulator until the tile ends.  The integers of the tile's
+// split are added by atomics, the same bits in any order.  lo grows by up to 2^40.4 a term: K <= 2^22 at once
+// (kDigitTerms).
 //
 // Layout.  The digits lie in memory as the tensor cores' K-major core matrices (8 rows x 16 bytes), ordered
 // [block of 32 k][digit][8 rows][4 x 8 k], so a tile's operand is seven contiguous pieces a stage, fetched by bulk
@@ -209,17 +218,21 @@ __device__ __forceinline__ bool tile_product(const Tile &t, unsigned char *smem,
         const int32_t chunk = it / kChunk;
         const bool first = it % kChunk == 0;
         const uint32_t a0 = smem_of(smem + s * kStageBytes), b0 = a0 + kDigits * kPieceA;
+        const auto pair = [&](int g, int i, bool fresh) {
+          for (int kk = 0; kk < kBK / 16; ++kk)
+            mma(tmem + g * kTN, operand(a0 + i * kPieceA + kk * 256), operand(b0 + (g - i) * kPieceB + kk * 256),
+                !(fresh && kk == 0));
+        };
         for (int g = 0; g < kDigits && ok; ++g) {
           if (first && chunk > 0) {
             ok = bar_wait(free_g + 8 * g, (chunk - 1) & 1);
             if (!ok) break;
             fence_after();
           }
-          for (int i = 0; i <= g; ++i)
-            for (int kk = 0; kk < kBK / 16; ++kk)
-              mma(tmem + g * kTN, operand(a0 + i * kPieceA + kk * 256), operand(b0 + (g - i) * kPieceB + kk * 256),
-                  !(first && i == 0 && kk == 0));
+          for (int i = 0; i <= g; ++i) pair(g, i, first && i == 0);
         }
+        if (!ok) break;
+        for (int i = 1; i < kDigits; ++i) pair(kDigits, i, it == 0 && i == 1);
         mma_commit(empty + 8 * s);
         if (it % kChunk == kChunk - 1 || it == stages - 1) mma_commit(done);
       }
@@ -229,7 +242,7 @@ __device__ __forceinline__ bool tile_product(const Tile &t, unsigned char *smem,
     const uint32_t base = tmem + ((uint32_t)(32 * quarter) << 16) + 32 * half;
     const int32_t chunks = (stages + kChunk - 1) / kChunk;
     for (int32_t c = 0; c < chunks; ++c) {
-      ok = bar_wait(done, c & 1);
+      ok = __all_sync(0xffffffffu, bar_wait(done, c & 1));  // the TMEM loads are the whole warp's
       if (!ok) break;
       fence_after();
 #pragma unroll
@@ -242,10 +255,16 @@ __device__ __forceinline__ bool tile_product(const Tile &t, unsigned char *smem,
 #pragma unroll
         for (int e = 0; e < 32; ++e) {
           const int32_t n = __float2int_rn(__uint_as_float(v[e]));
-          if (g < 3) hi[e] = mad(n, 1 << (8 * (2 - g)), hi[e]);
-          else lo[e] = mad(n, 1 << (8 * (6 - g)), lo[e]);
+          if (g < 4) hi[e] = mad(n, 1 << (8 * (3 - g)), hi[e]);
+          else lo[e] = mad(n, 1 << (8 * (7 - g)), lo[e]);
         }
       }
+    }
+    if (ok) {  // the last weight
+      uint32_t v[32];
+      tmem_load(base + kDigits * kTN, v);
+#pragma unroll
+      for (int e = 0; e < 32; ++e) lo[e] += __float2ll_rn(__uint_as_float(v[e]));
     }
   }
   __syncwarp();
@@ -300,7 +319,7 @@ __global__ void k_gram_finish(int32_t m, int32_t nn, int32_t mp, int32_t np, con
   const int32_t sp = mirror ? q : p, sq = mirror ? p : q;
   const int64_t at = (int64_t)sq * mp + sp;
   const int32_t a = ea[sp], b = eb[sq];
-  double v = to_double(acc[at], acc[at + (int64_t)mp * np], a == kNoExp || b == kNoExp ? 0 : a + b - 110 + 48);
+  double v = to_double(acc[at], acc[at + (int64_t)mp * np], a == kNoExp || b == kNoExp ? 0 : a + b - 110 + 40);
   if (a == kNotFinite || b == kNotFinite || *err) v = __longlong_as_double(0x7ff8000000000000ll);
   C[(int64_t)q * ldc + p] = alpha * v + (beta == 0.0 ? 0.0 : beta * C[(int64_t)q * ldc + p]);
 }
@@ -330,7 +349,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_update_digits(const uint16_t *A
       for (int e = 0; e < 32; ++e) {
         if (q0 + e >= N) break;
         const int32_t b = __ldg(eb + q0 + e);
-        double v = to_double(hi[e], lo[e], a == kNoExp || b == kNoExp ? 0 : a + b - 110 + 48);
+        double v = to_double(hi[e], lo[e], a == kNoExp || b == kNoExp ? 0 : a + b - 110 + 40);
         if (failed || a == kNotFinite || b == kNotFinite) v = __longlong_as_double(0x7ff8000000000000ll);
         c[e] = alpha * v + (beta == 0.0 ? 0.0 : beta * c[e]);
       }

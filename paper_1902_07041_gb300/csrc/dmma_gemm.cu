@@ -182,8 +182,10 @@ void launch_gram(int64_t K, int32_t m, int32_t nn, const double *A, int64_t lda,
                  DBuf *digits) {
   if (m <= 0 || nn <= 0) return;
   if (digits && (double)K * m * nn >= kGramDigits &&
-      room_for(*digits, digit_gram_bytes(K, m, nn, A == B && lda == ldb && m == nn))) {
-    launch_gram_digits(K, m, nn, A, lda, B, ldb, alpha, beta, C, ldc, sym, digits->p, s);
+      room_for(*digits, digit_gram_bytes(std::min(K, kDigitTerms), m, nn, A == B && lda == ldb && m == nn))) {
+    for (int64_t r0 = 0; r0 < K; r0 += kDigitTerms)
+      launch_gram_digits(std::min(K - r0, kDigitTerms), m, nn, A + r0 * lda, lda, B + r0 * ldb, ldb, alpha,
+                         r0 ? 1.0 : beta, C, ldc, sym, digits->p, s);
     return;
   }
   const int32_t splits = gram_splits(K, m, nn, sym);

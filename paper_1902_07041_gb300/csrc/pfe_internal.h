@@ -241,6 +241,7 @@ void launch_update(int64_t M, int32_t N, int32_t K, const double *A, int64_t lda
                    bool upper = false, DBuf *digits = nullptr);
 // With a buffer `digits` (grown as needed; without room the products stay on the FP64 path) large products run on the
 // BF16 tensor cores by exact digits (digit_gemm.cu).
+constexpr int64_t kDigitTerms = 1 << 22;  // contraction length whose digit sums 64 bits hold
 size_t digit_gram_bytes(int64_t K, int32_t m, int32_t nn, bool same);
 void launch_gram_digits(int64_t K, int32_t m, int32_t nn, const double *A, int64_t lda, const double *B, int64_t ldb,
                         double alpha, double beta, double *C, int64_t ldc, bool sym, void *work, cudaStream_t s);
