@@ -495,74 +495,119 @@ __device__ __forceinline__ int2 fixed_entry(double v, double unit) {
   return t > ((int64_t)1 << 61) - kHalf - 1 ? make_int2((int32_t)(t - ((int64_t)INT32_MAX << kLimb)), INT32_MAX) : split(t);
 }
 
+// *p = max(*p, v) for non-negative values, with an atomic only where it would change
+__device__ __forceinline__ void raise(int32_t *p, int32_t v) {
+  if (v > *reinterpret_cast<volatile int32_t *>(p)) atomicMax(p, v);
+}
 // info[0] |= 1 when the operator does not fit; info[1]: ||A||_inf as float bits, rounded up
 __device__ __forceinline__ void note_row(int32_t *info, double row, bool bad) {
   if (bad || !(row <= 16.0)) atomicOr(info, 1);
-  else atomicMax(info + 1, __float_as_int(__double2float_ru(row * 1.000001)));
+  else raise(info + 1, __float_as_int(__double2float_ru(row * 1.000001)));
+}
+// sums and maxima over the 16 lanes of an atom
+__device__ __forceinline__ double sum16(double v) {
+  for (int d = 8; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
+  return v;
+}
+__device__ __forceinline__ float max16(float v) {
+  for (int d = 8; d > 0; d >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, d));
+  return v;
+}
+__device__ __forceinline__ bool any16(bool v) {
+  return (__ballot_sync(0xffffffffu, v) >> (threadIdx.x & 16) & 0xffffu) != 0;
 }
 
+// Both kernels take 16 lanes an atom: with one a row's chain of FP64 conversions took 42 us at N = 800, as long as six
+// filter steps (10 us now), and a first call of few steps was slower than in the FP64 kernels.
+//
 // Rank-1 form, unit 2^-60.  With |x| < 2^60 the cross terms of a row's diagonal block and F of its other blocks
 // stay below 2^59 (3 + sum |d| + sum (|u_r| + |u|_1)), which 63 bits hold for a factor below 15.5: info[2], info[3]
 // get the largest one for F = 6, 4.  An operator whose factor for F = 2 is larger does not fit, nor does one with
 // |u|_1 >= 3.9 (the high limb of u . x would leave 32 bits, see top_of).  Neither occurs while the bound holds
 // (||A||_2 <= 2: |u|_2 <= sqrt(2), a diagonal row below 3.5).  info[4]: the longest row, info[5]: the largest |u|_1.
-__global__ void k_fixed_r1(int32_t n_atoms, const int32_t *__restrict__ rp1, const int32_t *__restrict__ ci1,
-                           const double *__restrict__ u, const double *__restrict__ dg, int4 *blk, int2 *dgo,
-                           int32_t *info) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n_atoms) return;
-  const double *d = dg + 6 * i;
-  double row[3] = {fabs(d[0]) + fabs(d[1]) + fabs(d[2]), fabs(d[1]) + fabs(d[3]) + fabs(d[4]),
-                   fabs(d[2]) + fabs(d[4]) + fabs(d[5])};
-  bool bad = !(row[0] < 4.0 && row[1] < 4.0 && row[2] < 4.0);
-  for (int t = 0; t < 6; ++t) {
-    bad = bad || !(fabs(d[t]) <= 2.0);
-    dgo[6 * i + t] = bad ? make_int2(0, 0) : fixed_entry(-d[t], 0x1p60);
-  }
-  const double drow = fmax(row[0], fmax(row[1], row[2]));
-  double s6[3] = {0, 0, 0}, s4[3] = {0, 0, 0}, s2[3] = {0, 0, 0}, m6 = 0.0, m4 = 0.0, m2 = 0.0, u1 = 0.0;
-  const int32_t p0 = rp1[i], p1 = rp1[i + 1];
-  for (int32_t p = p0; p < p1 && !bad; ++p) {
-    const double v[3] = {u[3 * (int64_t)p], u[3 * (int64_t)p + 1], u[3 * (int64_t)p + 2]};
-    const double s = fabs(v[0]) + fabs(v[1]) + fabs(v[2]);
-    if (!(fmax(fabs(v[0]), fmax(fabs(v[1]), fabs(v[2]))) < 1.99)) {  // a limb is 31 bits; |u|_2 <= sqrt(2) when ||A|| <= 2
-      bad = true;
-      break;
+// The factors are sums of floats, a relative 1e-5 up.  A pass takes 12 blocks, two groups of six, three of four.
+__global__ void __launch_bounds__(128) k_fixed_r1(int32_t n_atoms, const int32_t *__restrict__ rp1,
+                                                  const int32_t *__restrict__ ci1, const double *__restrict__ u,
+                                                  const double *__restrict__ dg, int4 *blk, int2 *dgo, int32_t *info) {
+  const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 4;
+  const int lane = threadIdx.x & 15;
+  const bool live = i < n_atoms;
+  double row[3] = {0.0, 0.0, 0.0};
+  float drow = 0.f;
+  bool bad = false;
+  if (live) {
+    double d[6];
+    for (int t = 0; t < 6; ++t) {
+      d[t] = dg[6 * i + t];
+      bad = bad || !(fabs(d[t]) <= 2.0);
     }
-    u1 = fmax(u1, s);
-    const bool new6 = (p - p0) % 6 == 0, new4 = (p - p0) % 4 == 0, new2 = (p - p0) % 2 == 0;
+    const double r[3] = {fabs(d[0]) + fabs(d[1]) + fabs(d[2]), fabs(d[1]) + fabs(d[3]) + fabs(d[4]),
+                         fabs(d[2]) + fabs(d[4]) + fabs(d[5])};
+    bad = bad || !(r[0] < 4.0 && r[1] < 4.0 && r[2] < 4.0);
+    drow = (float)fmax(r[0], fmax(r[1], r[2]));
+    if (lane == 0)
+      for (int t = 0; t < 3; ++t) row[t] = r[t];
+    if (lane < 6) dgo[6 * i + lane] = bad ? make_int2(0, 0) : fixed_entry(-dg[6 * i + lane], 0x1p60);
+  }
+  const int32_t p0 = live ? rp1[i] : 0, p1 = live ? rp1[i + 1] : 0;
+  const int32_t longest = max(p1 - p0, __shfl_xor_sync(0xffffffffu, p1 - p0, 16));  // of the warp's two atoms
+  float m6 = 0.f, m4 = 0.f, m2 = 0.f, u1 = 0.f;
+  for (int32_t at = 0; at < longest; at += 12) {
+    const int32_t p = p0 + at + lane;
+    float f[3] = {0.f, 0.f, 0.f};
+    if (lane < 12 && p < p1) {
+      const double v[3] = {u[3 * (int64_t)p], u[3 * (int64_t)p + 1], u[3 * (int64_t)p + 2]};
+      const double s = fabs(v[0]) + fabs(v[1]) + fabs(v[2]);
+      if (!(fmax(fabs(v[0]), fmax(fabs(v[1]), fabs(v[2]))) < 1.99 && s < 3.9)) {  // a limb is 31 bits (and see above)
+        bad = true;
+      } else {
+        u1 = fmaxf(u1, (float)s);
+        for (int r = 0; r < 3; ++r) {
+          row[r] += fabs(v[r]) * s;
+          f[r] = (float)(fabs(v[r]) + s);
+        }
+        const int2 a = fixed_entry(v[0], 0x1p60), b = fixed_entry(v[1], 0x1p60), c = fixed_entry(v[2], 0x1p60);
+        blk[2 * (int64_t)p] = make_int4(a.x, a.y, b.x, b.y);
+        blk[2 * (int64_t)p + 1] = make_int4(c.x, c.y, ci1[p], 0);
+      }
+    }
     for (int r = 0; r < 3; ++r) {
-      row[r] += fabs(v[r]) * s;
-      s6[r] = (new6 ? 0.0 : s6[r]) + fabs(v[r]) + s;
-      s4[r] = (new4 ? 0.0 : s4[r]) + fabs(v[r]) + s;
-      s2[r] = (new2 ? 0.0 : s2[r]) + fabs(v[r]) + s;
-      m6 = fmax(m6, s6[r]);
-      m4 = fmax(m4, s4[r]);
-      m2 = fmax(m2, s2[r]);
+      const float two = f[r] + __shfl_xor_sync(0xffffffffu, f[r], 1);
+      const float four = two + __shfl_xor_sync(0xffffffffu, two, 2);
+      const float six = two + __shfl_down_sync(0xffffffffu, two, 2, 16) + __shfl_down_sync(0xffffffffu, two, 4, 16);
+      m2 = fmaxf(m2, two);
+      m4 = fmaxf(m4, four);
+      if (lane == 0 || lane == 6) m6 = fmaxf(m6, six);
     }
-    const int2 a = fixed_entry(v[0], 0x1p60), b = fixed_entry(v[1], 0x1p60), c = fixed_entry(v[2], 0x1p60);
-    blk[2 * (int64_t)p] = make_int4(a.x, a.y, b.x, b.y);
-    blk[2 * (int64_t)p + 1] = make_int4(c.x, c.y, ci1[p], 0);
   }
-  bad = bad || !(u1 < 3.9 && 3.0 + drow + m2 < 15.5);
+  for (int r = 0; r < 3; ++r) row[r] = sum16(row[r]);
+  m6 = 1.00001f * (3.f + drow + max16(m6));
+  m4 = 1.00001f * (3.f + drow + max16(m4));
+  m2 = 1.00001f * (3.f + drow + max16(m2));
+  u1 = 1.00001f * max16(u1);
+  bad = any16(bad) || !(m2 < 15.5f);
+  if (!live || lane != 0) return;
   if (!bad) {
-    atomicMax(info + 2, __float_as_int((float)(3.0 + drow + m6)));
-    atomicMax(info + 3, __float_as_int((float)(3.0 + drow + m4)));
-    atomicMax(info + 5, __float_as_int((float)u1));
+    raise(info + 2, __float_as_int(m6));
+    raise(info + 3, __float_as_int(m4));
+    raise(info + 5, __float_as_int(u1));
   }
-  atomicMax(info + 4, p1 - p0);
+  raise(info + 4, p1 - p0);
   note_row(info, fmax(row[0], fmax(row[1], row[2])), bad);
 }
 
 // Full blocks, unit 2^-59: the cross terms of two blocks stay below 2^58 sum |a| + 2 x 3 2^59, which 63 bits hold
 // for ||A||_inf <= 16.
-__global__ void k_fixed_full(int32_t n_atoms, const int32_t *__restrict__ rp, const int32_t *__restrict__ ci,
-                             const double *__restrict__ A, int4 *blk, int32_t *info) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n_atoms) return;
+__global__ void __launch_bounds__(128) k_fixed_full(int32_t n_atoms, const int32_t *__restrict__ rp,
+                                                    const int32_t *__restrict__ ci, const double *__restrict__ A, int4 *blk,
+                                                    int32_t *info) {
+  const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 4;
+  const int lane = threadIdx.x & 15;
+  const bool live = i < n_atoms;
   double row[3] = {0.0, 0.0, 0.0};
   bool bad = false;
-  for (int32_t p = rp[i]; p < rp[i + 1] && !bad; ++p) {
+  const int32_t p0 = live ? rp[i] : 0, p1 = live ? rp[i + 1] : 0;
+  for (int32_t p = p0 + lane; p < p1; p += 16) {
     int2 v[10];
     for (int t = 0; t < 9; ++t) {
       const double e = A[9 * (int64_t)p + t];
@@ -573,7 +618,10 @@ __global__ void k_fixed_full(int32_t n_atoms, const int32_t *__restrict__ rp, co
     v[9] = make_int2(ci[p], 0);
     for (int t = 0; t < 5; ++t) blk[5 * (int64_t)p + t] = make_int4(v[2 * t].x, v[2 * t].y, v[2 * t + 1].x, v[2 * t + 1].y);
   }
-  atomicMax(info + 4, rp[i + 1] - rp[i]);
+  for (int r = 0; r < 3; ++r) row[r] = sum16(row[r]);
+  bad = any16(bad);
+  if (!live || lane != 0) return;
+  raise(info + 4, p1 - p0);
   note_row(info, fmax(row[0], fmax(row[1], row[2])), bad);
 }
 
@@ -731,7 +779,7 @@ size_t fixed_state_bytes(int64_t n, int32_t k) {
 
 void launch_fixed_operator(const Bsr<double> &A, void *blocks, void *diag, int32_t *info, cudaStream_t s) {
   cudaMemsetAsync(info, 0, kFixedInfo * sizeof(int32_t), s);
-  const unsigned grid = (unsigned)((A.n_atoms + 127) / 128);
+  const unsigned grid = (unsigned)((A.n_atoms + 7) / 8);  // 16 lanes an atom
   if (A.u)
     PFE_LAUNCH k_fixed_r1<<<grid, 128, 0, s>>>(A.n_atoms, A.rp1, A.ci1, A.u, A.dg, static_cast<int4 *>(blocks),
                                                static_cast<int2 *>(diag), info);

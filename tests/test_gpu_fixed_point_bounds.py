@@ -289,3 +289,22 @@ def test_adjoint_in_segments_gives_the_bits_of_one_segment(m, rank1):
         torch.cuda.empty_cache()
         for c, _ in ctxs:
             pfe.pfe_destroy(c)
+
+
+# rows around the 12 (rank-1) and 16 (full) blocks that a pass over the operator takes, and several passes
+@pytest.mark.parametrize("rank1,shape", [(1, 7), (0, 0)])
+@pytest.mark.parametrize("n", [2, 12, 13, 14, 17, 18, 40])
+def test_springs_between_all_pairs(n, rank1, shape):
+    rng = np.random.default_rng(n)
+    bi, bj = np.triu_indices(n, 1)
+    r = rng.standard_normal((bi.size, 3))
+    ctx = bonds_context(n, bi, bj, 1.0 + rng.random(bi.size), r / np.linalg.norm(r, axis=1)[:, None], 0.0)
+    try:
+        pfe.pfe_set_param(ctx, pfe.PFE_P_RANK1, rank1)
+        coef = np.cos(np.arange(8)) / (1.0 + np.arange(8))
+        X = rng.standard_normal((3 * n, 5))
+        Y, R = apply(ctx, coef, X), apply(ctx, coef, X, shape)
+        assert np.max(np.abs(Y - R)) <= tolerance(X, coef)
+        assert np.any(Y != R)  # rounded differently: the fixed-point form ran
+    finally:
+        pfe.pfe_destroy(ctx)
