@@ -104,8 +104,7 @@ enum {
   PFE_P_BLOCK = 22,         /* block size of METHOD 1 (default 64) */
   PFE_P_BASIS_FACTOR = 23,  /* METHOD 1: basis size = BASIS_FACTOR x the wanted count (default 2; >= 1.25) */
   PFE_P_BATCH_THREADS = 24, /* pfe_solve_batch, read from the first context: host threads that run the
-                               samples' set-up and dense steps concurrently, each sample on its own
-                               stream (0 = automatic: min(samples, hardware threads, 16); 1 = serial) */
+                               samples concurrently, each sample on its context's stream (0 = automatic: min(samples, hardware threads, 16); 1 = serial) */
   PFE_P_RANK1 = 25,         /* 1 (default): when every off-diagonal block of H is -k r r^T / sqrt(m_i m_j)
                                (a central-force network, eqs. (1)-(2)) the filter steps use that rank-1
                                form, 6 FMAs a block and column instead of 9; 0: always the full 3x3
@@ -348,19 +347,21 @@ pfe_status pfe_probe_fp64_fma(int32_t iters, int32_t reps, void *stream, double 
 
 /* Solve every context's interval problem; n_found[s] per sample.  Each context must have its
  * interval set; all must live on one device.  Samples whose filter runs in fixed point or in FP32
- * iterate independently, each on its own stream, from PFE_P_BATCH_THREADS host threads.  While some
+ * iterate independently, each on its context's stream, from PFE_P_BATCH_THREADS host threads.  Samples
+ * overlap on the device when their contexts were created on streams of their own; contexts created
+ * without one share the legacy default stream, and their kernels run one after another.  While some
  * sample's FP64 filter cannot run in fixed point (a forced kernel shape, degree 0, an operator that
  * does not fit), all samples advance in lockstep: the filters of those run as one persistent kernel
  * per Chebyshev step over their work, captured once in a CUDA graph and replayed per iteration (its
  * column tile and grid size chosen by timing the candidates on the first call), the rest per sample,
  * concurrently from the same threads.  When every context
  * selects PFE_P_METHOD = 1 the samples' block Lanczos solves run whole, concurrently from those
- * threads, each on its own stream, largest samples first; a finished sample's work buffers pass to
+ * threads, each on its context's stream, largest samples first; a finished sample's work buffers pass to
  * the next sample its thread solves (its eigenvectors stay), so only the solves in flight hold them
  * and none is freed while others run, and a sample that ran out of device memory beside the others
  * is solved again afterwards, alone.  All contexts of a batch select the same method (PFE_E_ARG otherwise).
  * In the stats of every sample seconds_filter is the batch's filter time: the shared launches' in
- * lockstep, else the longest of any sample.  In the subspace iteration too, a sample that ran out of
+ * lockstep, else the longest of any sample (on a shared stream with the other samples' kernels in between).  In the subspace iteration too, a sample that ran out of
  * device memory beside the others is solved again
  * after the batch, alone (its stats are then its own solve's), and every sample releases its work
  * buffers when the batch ends (its eigenvectors stay).

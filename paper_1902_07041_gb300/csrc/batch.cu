@@ -1,6 +1,6 @@
 // Batched solves of independent samples (the realisations of Sec. 4.2) in FP64 kernels, for batches with an
-// operator, degree or forced kernel shape that the fixed-point step does not take (the others iterate on their own
-// streams, see pfe_solve_batch): every sample's
+// operator, degree or forced kernel shape that the fixed-point step does not take (the others iterate on their
+// contexts' streams, see pfe_solve_batch): every sample's
 // filtered subspace iteration advances in lockstep, and the filter (Alg. 2) of all samples runs
 // as ONE persistent kernel per Chebyshev step.  Its warps walk a device-resident work list of
 // (sample, atom, column chunk) items, so samples of uneven size share the GPU evenly.  The m_max

@@ -1999,8 +1999,8 @@ pfe_status pfe_solve_batch(pfe_ctx **ctxs, int32_t nsamples, int32_t *n_found) {
   }
   if (any_bks && !all_bks) return pfe_fail(c0, PFE_E_ARG, "batch contexts must all select the same PFE_P_METHOD");
   if (all_bks) {
-    // block Lanczos samples: every sample's solve on its own stream, the samples concurrently from
-    // the host threads (their kernels overlap on the device); no shared graph
+    // block Lanczos samples: every sample's solve on its context's stream, the samples concurrently from
+    // the host threads (their kernels overlap on the device where the streams differ); no shared graph
     std::vector<int32_t> nf(nsamples, 0);
     // Work buffers (several n x basis blocks) pass from a finished sample to the next sample its host
     // thread solves, so that only the solves in flight hold them and no device memory is freed while
@@ -2072,7 +2072,7 @@ pfe_status pfe_solve_batch(pfe_ctx **ctxs, int32_t nsamples, int32_t *n_found) {
   };
   // set-up of every sample (filter design, width, buffers, start block); a sample that failed gives
   // back what it had reserved
-  // Samples whose filter runs in fixed point (or FP32) iterate on their own streams; the batched FP64 launches
+  // Samples whose filter runs in fixed point (or FP32) iterate on their contexts' streams; the batched FP64 launches
   // are for the rest.
   for_each_sample(c0->device, nsamples, nthreads, [&](int32_t i) {
     SolveState &st = ctxs[i]->solve;
@@ -2093,9 +2093,9 @@ pfe_status pfe_solve_batch(pfe_ctx **ctxs, int32_t nsamples, int32_t *n_found) {
   bool lockstep = false;
   for (int32_t i = 0; i < nsamples; ++i) lockstep = lockstep || ctxs[i]->solve.batched;
   if (!lockstep) {
-    // No sample waits for another: each runs all its iterations from one host thread, and the small launches of
-    // the samples overlap on the device.  Six glasses of 700 to 885 atoms: 195 ms in lockstep with the shared FP64
-    // launches, 187 ms this way (cuSOLVER's dense steps are most of it).
+    // Each sample runs all its iterations from one host thread, on its context's stream.  Six glasses of 700 to 885
+    // atoms: 100 ms with six streams, 190 ms where the contexts share the legacy default stream, on which nothing
+    // overlaps (195 ms in lockstep with the shared FP64 launches; 270 ms one after another).
     for_each_sample(c0->device, nsamples, nthreads, [&](int32_t i) {
       SolveState &st = ctxs[i]->solve;
       while (status[i] == PFE_OK && !st.done) {
