@@ -55,8 +55,12 @@ typedef enum {
 #define PFE_SKIP_SYM_CHECK 0x2u /* do not verify the symmetry of Delta */
 
 /* element types of pfe_filter_apply's X and Y */
-#define PFE_F64 0 /* float64 vectors, at least float64 accuracy (64-bit fixed point with a scale per column and
-                     step where the operator fits, else float64 arithmetic) */
+#define PFE_F64 0 /* float64 vectors.  Where the operator fits the recurrence runs in 64-bit fixed point with a scale
+                     per column and step: at least float64 accuracy in the norm of a column (60 bits below its
+                     largest entry, less log2(||Ht||_inf + 1)).  Entries far below a column's largest one, e.g. on a
+                     part of the network that is not connected with it, keep fewer bits than in float64
+                     arithmetic, none below 2^-57 of it; a forced kernel shape (PFE_P_STEP_SHAPE_F64) runs that.
+                     Else float64 arithmetic */
 #define PFE_F32 1 /* float32 vectors, float32 arithmetic (mixed-precision filter) */
 
 /* parameter keys for pfe_set_param / pfe_get_param (values are doubles) */

@@ -60,7 +60,8 @@ __device__ __forceinline__ int64_t shifted(int64_t v, int o) {
   if (o >= 0) return o > 62 ? 0 : (int64_t)((uint64_t)v << o);
   return o < -62 ? 0 : (v + ((int64_t)1 << (-o - 1))) >> -o;
 }
-// exact up to one rounding to double; two FP64 additions (the conversion instruction runs at 2 a clock as well)
+// Exact up to one rounding to double; two FP64 additions (the conversion instruction runs at 2 a clock as well).  The
+// two halves take the exponents 2^52 and 2^84, a known method (compiler-rt's __floatundidf).
 __device__ __forceinline__ double to_double(int64_t v) {
   const uint32_t lo = (uint32_t)v, hi = (uint32_t)((uint64_t)v >> 32) ^ 0x80000000u;
   const double dl = __hiloint2double(0x43300000, (int)lo);  // 2^52 + lo
@@ -296,10 +297,11 @@ struct ColumnScale {
 // atom and one group; its atoms' blocks (contiguous in the block list) and its columns' scales sit in shared
 // memory, so the neighbour loop's only global loads are the gathers, and passes > 1 spreads the set-up over
 // several atoms.
-// What bounds it: IMAD.WIDE runs at about 30 a clock and SM (measured), 18 a block and column make 165 us of the
-// step at N = 99,900, k = 64, and the moves and additions that share its pipe most of the rest (ncu: that pipe two
-// thirds busy); a step moves 614 MB there, 91 us at 6.76 TB/s.  Measured against the FP64 kernels: 876 -> 280 us a
-// step (k = 64), 13.8 -> 4.37 ms (k = 994), full blocks 250 -> 81 us (N = 20,000, k = 64).
+// What bounds it: the gathers' latency at 24 warps an SM, and the pipe of the multiplies.  IMAD.WIDE runs at about 30 a
+// clock and SM (measured), 18 a block and column make 165 us of the step at N = 99,900, k = 64; its pipe is 52 to 57 %
+// busy (ncu, N = 29,600, k = 64), with most stalls on the gathers.  A step moves 614 MB at N = 99,900, 91 us at 6.76
+// TB/s (ncu: DRAM 22 %, L2 20 % busy).  Measured against the FP64 kernels: 876 -> 280 us a step (k = 64), 13.8 -> 4.37 ms
+// (k = 994), full blocks 250 -> 81 us (N = 20,000, k = 64).
 // 24 warps an SM (80 registers).  Rank-1: CTAs of 128 lanes and one gather at a time; a second gather in flight
 // spills (303 us with 80 registers, 309 with 96), as do 64 registers (296).  Full blocks have three times the
 // products a gather and gain from it (81 against 89 us).  Prefetching rows to L1 or L2 only added instructions
