@@ -78,7 +78,9 @@ enum {
                                FP32 while its residual exceeds REFINE_TOL, in FP64 after; 2 mixed by defect
                                correction: as 1, but below REFINE_TOL the pair's filter is split exactly into
                                x p(theta) in FP64 plus a recurrence on its residual H x - theta x in FP32 (no
-                               FP64 filter sweep); the dense steps and residuals are FP64 in every mode */
+                               FP64 filter sweep); the dense steps and residuals are FP64 in every mode (large
+                               products by exact 8-bit digits: an FP64 sum's accuracy relative to the columns'
+                               largest entries) */
   PFE_P_MAX_ITERS = 9,      /* subspace-iteration limit (default 60) */
   PFE_P_SEED = 10,          /* seed of the random start block and estimator vectors (default 0) */
   PFE_P_LAMBDA_MAX = 11,    /* spectrum upper bound; 0 = estimate by Lanczos (default 0) */

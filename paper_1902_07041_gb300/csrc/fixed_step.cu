@@ -973,7 +973,8 @@ size_t fixed_adjoint_state_bytes(int64_t n, int32_t k, int32_t m, int32_t seg) {
 }
 
 // One segment keeps every t_j and a_j: 2 m steps.  More recompute the t_j of each from a saved pair (with its exponents,
-// so that they are the same bits), up to 3 m steps: N = 20,000, k = 32, m = 60 takes 14.7 ms with one segment.
+// so that they are the same bits), up to 3 m steps.  N = 20,000, k = 64, m = 200: 79 ms with one segment (12.4 GB), 87
+// with three (4.4 GB), 155 in the FP64 kernels; N = 50,000, k = 64, m = 60: 55, 61 and 109 ms.
 const double *launch_fixed_adjoint(const Bsr<double> &A, const FixedOp &op, const double *coef, int32_t m, int32_t seg,
                                    int32_t k, int64_t ld, const double *X, int64_t ldx, const double *Ybar, int64_t ldyb,
                                    int64_t nnzb, double two_over_d, double *vals_bar, double *work, void *state,

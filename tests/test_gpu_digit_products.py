@@ -136,6 +136,39 @@ def test_gram_of_zero_and_not_finite_columns(lib):
     assert not G[3, ~bad].any() and np.isfinite(G[np.ix_(~bad, ~bad)]).all()
 
 
+class DBuf(ctypes.Structure):
+    """The library's growing device buffer."""
+    _fields_ = [("p", P), ("bytes", ctypes.c_size_t)]
+
+
+@pytest.mark.parametrize("sym", [False, True])
+def test_gram_longer_than_its_sums(lib, sym):
+    """More rows than 64-bit sums hold at once: the dispatch adds two parts, each rounded to double."""
+    f = lib._ZN3pfe11launch_gramEliiPKdlS1_lddPdlbS2_P11CUstream_stPNS_4DBufE
+    f.restype, f.argtypes = None, [L, I, I, P, L, P, L, D, D, P, L, B, P, P, P]
+    free = lib._ZN3pfe9dbuf_freeERNS_4DBufE
+    free.restype, free.argtypes = None, [P]
+    size = lib._ZN3pfe9gram_workEliib
+    size.restype, size.argtypes = ctypes.c_size_t, [L, I, I, B]
+    K, m = (1 << 22) + 1000, 3
+    work = torch.empty(size(K, m, m, sym), dtype=torch.float64, device="cuda")
+    A, C = block("normal", K, m, 11), block("normal", m, m, 12)
+    C = C + C.T
+    a, c, buf = torch.from_numpy(A).cuda(), torch.from_numpy(C.copy()).cuda(), DBuf()
+    torch.cuda.synchronize()
+    f(K, m, m, a.data_ptr(), m, a.data_ptr(), m, 1.0, 0.5, c.data_ptr(), m, sym, work.data_ptr(), None,
+      ctypes.byref(buf))
+    torch.cuda.synchronize()
+    assert buf.bytes > 0  # the digits' workspace: that path ran
+    free(ctypes.byref(buf))
+    G = c.cpu().numpy().T
+    for i in range(m):
+        for j in range(m):
+            v = dot(A[:, i], A[:, j])
+            bound = gram_bound(A[:, i], A[:, j], v) + 2.0**-51 * (abs(v) + abs(C[i, j]))
+            assert abs(G[i, j] - (v + 0.5 * C[i, j])) <= bound, (i, j)
+
+
 def update(lib, A, Bm, alpha=1.0, beta=0.0, C=None, upper=False):
     """alpha A B + beta C, A and C row-major, B column-major."""
     M, K = A.shape
