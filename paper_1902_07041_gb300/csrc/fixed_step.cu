@@ -951,7 +951,8 @@ void launch_fixed_filter(const Bsr<double> &A, const FixedOp &op, const double *
 namespace {
 
 __global__ void k_copy16(int64_t words, const int4 *__restrict__ a, int4 *__restrict__ b) {
-  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < words; t += (int64_t)gridDim.x * blockDim.x) b[t] = a[t];
+  const int64_t all = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < words; t += all) b[t] = a[t];
 }
 void copy16(const void *a, void *b, int64_t words, cudaStream_t s) {
   PFE_LAUNCH k_copy16<<<(unsigned)std::min<int64_t>((words + 255) / 256, 4096), 256, 0, s>>>(

@@ -308,3 +308,47 @@ def test_springs_between_all_pairs(n, rank1, shape):
         assert np.any(Y != R)  # rounded differently: the fixed-point form ran
     finally:
         pfe.pfe_destroy(ctx)
+
+
+def test_solves_with_a_row_too_long_for_the_fixed_point_step():
+    """An atom with 790 weak springs: its row does not fit a CTA's shared memory.  Alone and in a batch beside a network
+    that fits, the solves take the FP64 kernels for it and find what LAPACK finds."""
+    g = glassgen.generate(800, 12)
+    rng = np.random.default_rng(1)
+    near = set(g.bj[g.bi == 0]) | set(g.bi[g.bj == 0])
+    far = np.array([j for j in range(1, 800) if j not in near], np.int32)
+    r = rng.standard_normal((far.size, 3))
+    bi, bj = np.r_[g.bi, np.zeros_like(far)], np.r_[g.bj, far]
+    ks = np.r_[g.k, 1e-4 * g.k.mean() * np.ones(far.size)]
+    rhat = np.r_[g.rhat, r / np.linalg.norm(r, axis=1)[:, None]]
+    nets = [(bi, bj, ks, rhat), (g.bi, g.bj, g.k, g.rhat)]
+    ctxs = []
+    try:
+        exact = []
+        for t in nets:
+            rp, ci, vals = pfe.pfe_springs_to_bsr(800, *t)
+            ctxs.append(pfe.pfe_create(800, rp, ci, vals, g.mass))
+            H = np.zeros((2400, 2400))
+            for i in range(800):
+                for p in range(rp[i], rp[i + 1]):
+                    blk = vals[9 * p:9 * p + 9].reshape(3, 3) / np.sqrt(g.mass[i] * g.mass[ci[p]])
+                    H[3 * i:3 * i + 3, 3 * ci[p]:3 * ci[p] + 3] = blk
+            w = np.linalg.eigvalsh(H)
+            a, b = 0.5 * (w[40] + w[41]), 0.5 * (w[80] + w[81])
+            pfe.pfe_set_interval(ctxs[-1], a, b)
+            exact.append(w[41:81])
+        assert np.diff(pfe.pfe_springs_to_bsr(800, *nets[0])[0]).max() - 1 > 768
+        for batch in (False, True):
+            if batch:
+                found, status = pfe.pfe_solve_batch(ctxs)
+                assert status == pfe.PFE_OK
+            else:
+                found = [pfe.pfe_solve(c)[0] for c in ctxs]
+                shapes = [pfe.pfe_get_stats(c)["filter_shape_f64"] for c in ctxs]
+                assert shapes[0] != 12 and shapes[1] == 12
+            for c, nf, w in zip(ctxs, found, exact):
+                lam, _, _ = pfe.pfe_get_eigenpairs(c, 2400, nf)
+                assert nf == 40 and np.allclose(lam, w, rtol=1e-10, atol=0)
+    finally:
+        for c in ctxs:
+            pfe.pfe_destroy(c)
